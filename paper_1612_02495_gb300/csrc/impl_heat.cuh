@@ -40,9 +40,10 @@ SchemeImpl make_heat() {
   return im;
 }
 
+template <typename T = double>  // a template: only the FP64 unit instantiates its kernels
 SchemeImpl make_heat_f64() {
-  using A = AdjLaunch<double, HeatAdjOp<double>>;
-  SchemeImpl im = make_heat<double>();
+  using A = AdjLaunch<T, HeatAdjOp<T>>;
+  SchemeImpl im = make_heat<T>();
   im.make_adj_consts = heat_adj_consts;
   im.adj_prepare = A::prepare;
   im.adj_up = A::up;

@@ -4,7 +4,7 @@
 namespace swept {
 
 const SchemeImpl* heat_impl_f64() {
-  static const SchemeImpl k = make_heat_f64();
+  static const SchemeImpl k = make_heat_f64<>();
   return &k;
 }
 

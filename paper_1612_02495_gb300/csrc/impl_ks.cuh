@@ -48,9 +48,10 @@ SchemeImpl make_ks() {
   return im;
 }
 
+template <typename T = double>  // a template: only the FP64 unit instantiates its kernels
 SchemeImpl make_ks_f64() {
-  using A = AdjLaunch<double, KsAdjOp<double>>;
-  SchemeImpl im = make_ks<double>();
+  using A = AdjLaunch<T, KsAdjOp<T>>;
+  SchemeImpl im = make_ks<T>();
   im.make_adj_consts = ks_adj_consts;
   im.adj_prepare = A::prepare;
   im.adj_up = A::up;

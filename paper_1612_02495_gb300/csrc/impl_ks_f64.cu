@@ -4,7 +4,7 @@
 namespace swept {
 
 const SchemeImpl* ks_impl_f64() {
-  static const SchemeImpl k = make_ks_f64();
+  static const SchemeImpl k = make_ks_f64<>();
   return &k;
 }
 

@@ -114,10 +114,7 @@ __device__ __forceinline__ void paired_level(T* sm, int M, int out_row, int lo, 
 template <typename T, class Op, int STAGE>
 __device__ __forceinline__ void scalar_level_any(T* sm, int M, int out_row, int lo, int hi, int wall, int chunk,
                                                  const typename Op::K& k) {
-  // FP32 only: in FP64 a warp instruction holds the FP64 pipe for 64 cycles
-  // whatever its active lanes, and pairs double the partial-warp waste at the
-  // triangle tips (measured 4 % slower on the FP64 KS workload)
-  if constexpr (Op::R == 2 && sizeof(T) == 4) {
+  if constexpr (Op::R == 2) {
     if (wall == NO_WALL && chunk <= 1 && ((lo | hi | M) & 1) == 0) {
       paired_level<T, Op, STAGE>(sm, M, out_row, lo, hi, k);
       return;
@@ -301,6 +298,55 @@ struct LevelImpl {
       scalar_level_any<T, Op, 0>(sm, M, out_row, lo, hi, wall, chunk, k);
     else
       scalar_level_any<T, Op, 1>(sm, M, out_row, lo, hi, wall, chunk, k);
+  }
+};
+// KS in FP64: a tier's points on the integer and FP64 pipes together
+// (KsOp::point_int).  KS grids are periodic, so a window never holds a wall,
+// and chunk 2 has nothing to gain: one point already keeps both pipes busy.  A
+// point the integer arithmetic does not handle is left out in the first loop
+// and redone in FP64 after it (under 1 % of the warps on the KS workload), so
+// that the loop has no branch and a warp's FP64 instructions start before its
+// integer chain has ended: with the branch at each point a lone warp took 1190
+// cycles a point, without 929.
+// Bound: FP64 and integer issue (58 % and 65 % of their pipes).  2^20 points,
+// tile 1024, 256 threads, persistent, 1,000 steps: 44.6 -> 26.0 ms.  Two points
+// a thread, sharing their operands' conversions, gave 25.3 ms there but took
+// 2^14 points (tile 128) from 3.85 to 4.22 ms (start: 4.06 ms); four spilled (36.6 ms); four or
+// five blocks a SM instead of three 27.2 and 28.3 ms.
+template <int STAGE>
+__device__ __noinline__ void ks_f64_redo(const double* in, double* out, int lo, int hi, KsOp<double>::K k) {
+  for (int j = lo + (int)threadIdx.x; j < hi; j += (int)blockDim.x) {
+    const double p2 = STAGE == 1 ? out[j] : 0.0;
+    double r;
+    if (!KsOp<double>::point_int<STAGE>(in + j - 2, p2, k, r)) out[j] = KsOp<double>::point_fp<STAGE>(in + j - 2, p2, k);
+  }
+}
+template <int STAGE>
+__device__ __forceinline__ void ks_f64_level(double* sm, int M, int out_row, int lo, int hi,
+                                             const KsOp<double>::K& k) {
+  const double* in = sm + (out_row ^ 1) * M;
+  double* out = sm + out_row * M;
+  bool bad = false;
+  for (int j = lo + (int)threadIdx.x; j < hi; j += (int)blockDim.x) {
+    double v[5];
+#pragma unroll
+    for (int d = 0; d < 5; ++d) v[d] = in[j + d - 2];
+    const double p2 = STAGE == 1 ? out[j] : 0.0;
+    double r;
+    const bool ok = KsOp<double>::point_int<STAGE>(v, p2, k, r);
+    if (ok) out[j] = r;
+    bad = bad || !ok;
+  }
+  if (bad) ks_f64_redo<STAGE>(in, out, lo, hi, k);
+}
+template <>
+struct LevelImpl<double, KsOp<double>> {
+  __device__ __forceinline__ static void run(double* sm, int M, int stage, int out_row, int lo, int hi, int /*wall*/,
+                                             int /*chunk*/, const KsOp<double>::K& k) {
+    if (stage == 0)
+      ks_f64_level<0>(sm, M, out_row, lo, hi, k);
+    else
+      ks_f64_level<1>(sm, M, out_row, lo, hi, k);
   }
 };
 // Euler: chunk 2 = two threads per face in the flux phase
@@ -492,7 +538,7 @@ struct RegCtx : Base {
     if (wall == NO_WALL) {
 #pragma unroll
       for (int i = 0; i < P; ++i) {
-        const T r = Op::template point<STAGE>(&w[i], dst[i], this->k);
+        const T r = Op::template point_fp<STAGE>(&w[i], dst[i], this->k);
         if (p0 + i >= lo && p0 + i < hi) dst[i] = r;
       }
     } else {
@@ -510,7 +556,7 @@ struct RegCtx : Base {
             if (q == e - R) x = w[i + e];
           v[d] = x;
         }
-        const T r = Op::template point<STAGE>(v, dst[i], this->k);
+        const T r = Op::template point_fp<STAGE>(v, dst[i], this->k);
         if (p0 + i >= lo && p0 + i < hi) dst[i] = r;
       }
     }

@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fixadd.cuh"
 #include "swept_geom.cuh"
 
 namespace swept {
@@ -39,9 +40,13 @@ struct HeatOp {
   };
   // v[0..2] = T_{i-1}, T_i, T_{i+1} at the previous tier
   template <int STAGE>
-  __device__ __forceinline__ static T point(const T* v, T /*prev2*/, const K& k) {
+  __device__ __forceinline__ static T point_fp(const T* v, T /*prev2*/, const K& k) {
     const T s = add_rn(v[2], v[0]);
     return fma_rn(k.fo, s, mul_rn(k.c1, v[1]));
+  }
+  template <int STAGE>
+  __device__ __forceinline__ static T point(const T* v, T prev2, const K& k) {
+    return point_fp<STAGE>(v, prev2, k);
   }
 };
 
@@ -61,19 +66,51 @@ struct KsOp {
   struct K {
     T ca, c2, c4, mdth, mdt;
   };
+  // the common end of g: from u_{i+1}, u_{i-1}^2 and the two differences
+  __device__ __forceinline__ static T combine(T up, T um2, T d2, T d4, const K& k) {
+    return fma_rn(k.c4, d4, fma_rn(k.c2, d2, mul_rn(k.ca, fma_rn(up, up, -um2))));
+  }
   __device__ __forceinline__ static T g(const T* v, const K& k) {
     const T sp1 = add_rn(v[3], v[1]);
     const T sp2 = add_rn(v[4], v[0]);
-    const T nl = fma_rn(v[3], v[3], -mul_rn(v[1], v[1]));
     const T d2 = fma_rn(T(-2), v[2], sp1);
     const T d4 = fma_rn(T(6), v[2], fma_rn(T(-4), sp1, sp2));
-    return fma_rn(k.c4, d4, fma_rn(k.c2, d2, mul_rn(k.ca, nl)));
+    return combine(v[3], mul_rn(v[1], v[1]), d2, d4, k);
   }
-  // v[0..4] = u_{i-2} .. u_{i+2} at the previous tier; prev2 = u_i two tiers back
+  // v[0..4] = u_{i-2} .. u_{i+2} at the previous tier; prev2 = u_i two tiers back.
+  // point_fp: every operation on the floating-point pipes.
+  template <int STAGE>
+  __device__ __forceinline__ static T point_fp(const T* v, T prev2, const K& k) {
+    return fma_rn(STAGE == 0 ? k.mdth : k.mdt, g(v, k), STAGE == 0 ? v[2] : prev2);
+  }
+  // FP64: the sums, differences and the square on the integer pipes (fixadd.cuh),
+  // five of the eleven operations on the FP64 pipe.  False (r meaningless) where
+  // the integer arithmetic does not handle an operand; the caller then takes
+  // point_fp, behind a real branch: a FP64 instruction whose guard predicate is
+  // false holds the pipe as long as one that runs (77 cycles).
+  template <int STAGE>
+  __device__ __forceinline__ static bool point_int(const T* v, T prev2, const K& k, T& r) {
+    T d2, d4, um2;
+    const bool lin = fix::second_fourth(v[0], v[1], v[2], v[3], v[4], d2, d4);
+    const bool sq = fix::square(v[1], um2);
+    r = fma_rn(STAGE == 0 ? k.mdth : k.mdt, combine(v[3], um2, d2, d4, k), STAGE == 0 ? v[2] : prev2);
+    return lin && sq;
+  }
+  // the FP64 instructions out of line: a call is never turned into predicated instructions
+  template <int STAGE>
+  __device__ __noinline__ static T point_cold(T a, T b, T c, T d, T e, T prev2, K k) {
+    const T v[5] = {a, b, c, d, e};
+    return point_fp<STAGE>(v, prev2, k);
+  }
   template <int STAGE>
   __device__ __forceinline__ static T point(const T* v, T prev2, const K& k) {
-    if (STAGE == 0) return fma_rn(k.mdth, g(v, k), v[2]);
-    return fma_rn(k.mdt, g(v, k), prev2);
+    if constexpr (sizeof(T) == 8) {
+      T r;
+      if (!point_int<STAGE>(v, prev2, k, r)) r = point_cold<STAGE>(v[0], v[1], v[2], v[3], v[4], prev2, k);
+      return r;
+    } else {
+      return point_fp<STAGE>(v, prev2, k);
+    }
   }
 };
 
