@@ -109,6 +109,12 @@ typedef enum {
  *            shared-memory access and no barrier.
  *            Works with the per-pass, persistent and cluster modes; results are
  *            bit-identical to the shared-memory tiers.
+ * When tile_w, threads, chunk, persistent, cluster and warp_tiles are all 0, the library also
+ * chooses the decomposition: swept_step_n keeps a small heat or KS grid (up to
+ * a few thousand points in FP64, tens of thousands in FP32) in the registers of
+ * one thread-block cluster for the whole solve, with ghost points traded every
+ * few sub-timesteps.  The values are the same bit for bit, and the plan report
+ * still describes the tiles that the other calls use.
  * Stability (Fo <= 1/2, CFL) is the caller's responsibility and is not checked.
  */
 typedef struct {

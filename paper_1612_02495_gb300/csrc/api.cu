@@ -71,6 +71,45 @@ int choose_tile(int64_t n, int R, int sms) {
   return 0;
 }
 
+// The resident kernel (resident.cuh) for an n-point grid, or P = 0 where the
+// swept passes are the faster choice.  Cycles per sub-timestep: a warp alone
+// needs its shuffles and its dependent chain (28 + `chain`) and issues `ops`
+// operations per point (64 cycles each in FP64, where a warp instruction holds
+// the pipe that long); m warps share a sub-partition; a trade costs 700 cycles
+// across a cluster and 100 within a block, every `tiers` sub-timesteps.  The
+// smallest sum over points per lane, warps and blocks is taken; it came out 10
+// to 30 cycles below what was measured.  Beyond `limit` the swept passes are
+// faster.  Measured cycles per sub-timestep, resident against the default tile:
+//   heat FP32  1024: 94 / 2420   8192: 94 / 958    32768: 150 / 621
+//   heat FP64  1024: 373 / 2706  4096: 843 / 1790  8192: 1477 / 1303
+//   KS FP32    1024: 134 / 2357  8192: 175 / 1422  16384: 264 / 977  32768: 393 / 742
+//   KS FP64    1024: 1061 / 3113 4096: 2692 / 3206 8192: 4756 / 2541
+swept::ResidentPlan choose_resident(int64_t n, const SchemeImpl* im) {
+  swept::ResidentPlan best;
+  if (!im->resident || n > 65536) return best;
+  const bool f64 = im->value_bytes == 8;
+  const int ops = im->R == 1 ? 3 : 11, N = (int)n;
+  const double per_op = f64 ? 64.0 : 1.0, chain = f64 ? 64.0 : (im->R == 1 ? 8.0 : 25.0);
+  const double limit = f64 ? (im->R == 1 ? 1000.0 : 2600.0) : 350.0;
+  double best_t = limit;
+  for (int P = 1; P <= 8; P *= 2)
+    for (int blocks = 1; blocks <= 16; blocks *= 2)
+      for (int warps = 1; warps <= 16; ++warps) {
+        const int own = (N + blocks * warps - 1) / (blocks * warps), ghost = (32 * P - own) / 2;
+        int tiers = std::min(64, ghost / im->R);
+        tiers -= tiers % im->S;
+        if (own < 1 || tiers < std::max(2, im->S)) continue;
+        const int m = (warps + 3) / 4;
+        const double issue = P * ops * per_op + 4 * im->R + 4;
+        const double t = std::max(28.0 + chain + P * ops * per_op, m * issue) + (blocks > 1 ? 700.0 : 100.0) / tiers;
+        if (t < best_t) {
+          best_t = t;
+          best = swept::ResidentPlan{P, warps, blocks, own, tiers};
+        }
+      }
+  return best;
+}
+
 swept_status no_tiling(swept_handle* h) {
   return fail(h, SWEPT_EUNSUPPORTED, "grid too small for a swept tiling (fewer than two tiles of 4r points): "
                                      "only classic_step_n runs on this handle");
@@ -417,6 +456,10 @@ swept_status swept_init(const swept_config* cfg, swept_handle** out) {
     delete h;
     return SWEPT_EINVAL;
   }
+  // the whole plan left to the library: small grids stay on chip for the whole solve
+  if (h->tiled && cfg->tile_w == 0 && cfg->threads == 0 && cfg->chunk == 0 && !h->persistent && !h->cluster &&
+      cfg->warp_tiles == 0)
+    h->resident = choose_resident(cfg->n, im);
   (void)e;
   *out = h;
   return SWEPT_OK;
@@ -450,6 +493,16 @@ swept_status swept_step_n(swept_handle* h, void* u_dev, int64_t nsteps, void* st
   if (nsteps == 0) return st;
   const cudaStream_t s = (cudaStream_t)stream;
   const int64_t n_sub = nsteps * h->g.S;
+  if (h->resident.P && !h->resident_checked) {
+    // a cluster this size may not be schedulable (a partitioned GPU): then the swept passes
+    if (!h->impl->resident_fits(h->resident)) h->resident.P = 0;
+    cudaGetLastError();
+    h->resident_checked = true;
+  }
+  if (h->resident.P) {
+    const cudaError_t e = h->impl->resident(h->g, h->k, u_dev, n_sub, h->resident, s);
+    return e == cudaSuccess ? SWEPT_OK : cuda_fail(h, e, "resident kernel");
+  }
   if (h->cluster) {
     return run_graph(h, key_of("swept_cluster", u_dev, nsteps), s, [&](cudaStream_t cs) {
       return h->impl->cluster(h->g, h->k, u_dev, n_sub, h->threads, h->smem, cs);

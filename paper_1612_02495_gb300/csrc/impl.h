@@ -12,6 +12,12 @@ namespace swept {
 
 constexpr int KBYTES = 64;  // room for any scheme's constant struct
 
+// resident kernel: points per lane, warps per block, blocks of the cluster,
+// points a warp owns, sub-timesteps between trades (0 points: not used)
+struct ResidentPlan {
+  int P = 0, warps = 0, blocks = 0, own = 0, tiers = 0;
+};
+
 struct SchemeImpl {
   int R, S, C;
   int value_bytes;
@@ -60,6 +66,11 @@ struct SchemeImpl {
                          int hh, int write_top, int threads, size_t smem, cudaStream_t s);
   cudaError_t (*slab_diamond)(const Geom& g, const Slab& sl, const void* k, void* u_out, const void* e_in,
                               void* e_out, int odd, int mode, int hh, int threads, size_t smem, cudaStream_t s);
+  // the whole solve with the grid in the registers of one thread-block
+  // cluster (resident.cuh); nullptr where there is none
+  cudaError_t (*resident)(const Geom& g, const void* k, void* u, int64_t n_sub, const ResidentPlan& r,
+                          cudaStream_t s);
+  bool (*resident_fits)(const ResidentPlan& r);  // a cluster of that size can run on the current device
 };
 
 // Raise kernel `fn`'s dynamic shared-memory limit on the current device to at

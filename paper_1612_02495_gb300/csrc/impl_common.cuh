@@ -6,6 +6,7 @@
 
 #include "impl.h"
 #include "kernels.cuh"
+#include "resident.cuh"
 
 namespace swept {
 
@@ -146,6 +147,58 @@ struct Launch {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, fn, g, kc(k), (T*)u, n_sub, win_values);
+  }
+  // fn(std::integral_constant<int, P>) for the resident kernel of P points a lane
+  template <class Fn>
+  static cudaError_t with_resident(int P, Fn&& fn) {
+    switch (P) {
+      case 1: return fn(std::integral_constant<int, 1>{});
+      case 2: return fn(std::integral_constant<int, 2>{});
+      case 4: return fn(std::integral_constant<int, 4>{});
+      case 8: return fn(std::integral_constant<int, 8>{});
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  // launch configuration of the resident kernel `fn`; attr is the caller's
+  static cudaError_t resident_config(const void* fn, const ResidentPlan& r, cudaStream_t s, cudaLaunchAttribute* attr,
+                                     cudaLaunchConfig_t* cfg) {
+    const size_t bytes = 2 * (size_t)r.warps * r.own * sizeof(T);
+    cudaError_t e = raise_smem_limit(fn, bytes);
+    if (e == cudaSuccess && r.blocks > 8)
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cfg->gridDim = dim3((unsigned)r.blocks, 1, 1);
+    cfg->blockDim = dim3((unsigned)(32 * r.warps), 1, 1);
+    cfg->dynamicSmemBytes = bytes;
+    cfg->stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)r.blocks;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+    return e;
+  }
+  static cudaError_t resident(const Geom& g, const void* k, void* u, int64_t n_sub, const ResidentPlan& r,
+                              cudaStream_t s) {
+    return with_resident(r.P, [&](auto pc) {
+      auto fn = k_resident<T, Op, decltype(pc)::value>;
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute attr;
+      const cudaError_t e = resident_config((const void*)fn, r, s, &attr, &cfg);
+      if (e != cudaSuccess) return e;
+      return cudaLaunchKernelEx(&cfg, fn, (int)g.N, g.bc, kc(k), (T*)u, n_sub, r.own, r.tiers);
+    });
+  }
+  static bool resident_fits(const ResidentPlan& r) {
+    int n = 0;
+    const cudaError_t e = with_resident(r.P, [&](auto pc) {
+      auto fn = k_resident<T, Op, decltype(pc)::value>;
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute attr;
+      const cudaError_t e2 = resident_config((const void*)fn, r, nullptr, &attr, &cfg);
+      return e2 == cudaSuccess ? cudaOccupancyMaxActiveClusters(&n, fn, &cfg) : e2;
+    });
+    return e == cudaSuccess && n > 0;
   }
   static cudaError_t slab_prepare(size_t bytes) {
     cudaError_t e = raise_smem_limit((const void*)k_slab_up<T, Op>, bytes);

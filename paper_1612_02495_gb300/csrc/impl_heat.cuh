@@ -37,6 +37,8 @@ SchemeImpl make_heat() {
   im.slab_prepare = L::slab_prepare;
   im.slab_up = L::slab_up;
   im.slab_diamond = L::slab_diamond;
+  im.resident = L::resident;
+  im.resident_fits = L::resident_fits;
   return im;
 }
 

@@ -28,6 +28,8 @@ struct swept_handle {
   bool tiled = true;  // false: the grid is too small for a swept tiling (classic only)
   bool persistent = false;
   bool cluster = false;
+  swept::ResidentPlan resident;  // P > 0: swept_step_n runs the resident kernel
+  bool resident_checked = false;   // its cluster size is known to be schedulable
   int persist_blocks = 0;  // co-resident blocks of the persistent kernel (0 = not yet queried)
   uint32_t spin_limit = 1u << 24;  // polls a persistent block waits for an input tile (swept_set_option)
   int64_t start_item = 0;          // first queue item the persistent kernel claims (swept_set_option)
