@@ -89,7 +89,9 @@ typedef enum {
  *   chunk    heat and KS: 1 = one point per thread per trip through a tier
  *            (strided; in FP32, radius-2 tiers take aligned pairs of points,
  *            the default); 2 = two strided points (j, j + threads) with both
- *            windows loaded first.  Euler: 1 = one thread per face in the flux
+ *            windows loaded first.  FP32 tiles of up to 8 points per thread (4 in
+ *            the persistent and cluster modes) and all FP64 KS tiers have one
+ *            mapping of their own, which both values select.  Euler: 1 = one thread per face in the flux
  *            phase of a tier; 2 = two threads per face (one per reconstructed
  *            side, exchanged by warp shuffle)
  *   persistent 0: one kernel launch per swept pass (graph-captured); 1: the

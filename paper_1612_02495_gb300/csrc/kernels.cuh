@@ -369,6 +369,112 @@ struct LevelImpl<T, EulerOp<T>> {
 };
 
 // ---------------------------------------------------------------------------
+// FP32 tiers of the scalar schemes, all tiers of a phase with a fixed mapping
+// of points to threads: thread t owns the aligned pairs at J0 + 2 (t + q T),
+// q < Q, of the window and keeps both tier rows of its pairs in registers.  A
+// tier reads the two neighbouring pairs from shared memory, takes its own and
+// the value two tiers back from registers, and stores the pair for its
+// neighbours.  Addresses are loop invariant and a pair costs one range test, so
+// a tier alone takes about 230 cycles where the mapping that starts at the
+// tier's first point, recomputes its addresses and reloads its own pair takes
+// 330.  Bound: that latency on small tiles, instruction issue on large ones (11 of
+// about 20 instructions a KS point are arithmetic; whole warps at a
+// range's two ends).  Measured, before and after: KS 65,537 points, 2,000 steps 1.29 -> 0.93
+// ms; KS 2^20, tile 1024, 128 threads, 5,000 steps 7.71 -> 7.44; heat 2^20,
+// tile 256, 128 threads, 1,000 steps 1.26 -> 0.90; a batch of 128 problems 4.41 -> 3.50.
+// ---------------------------------------------------------------------------
+template <class Op, int Q, bool ODD>
+struct FixedTiers {
+  static constexpr int R = Op::R, J0 = R & ~1;
+  using K = typename Op::K;
+
+  template <int STAGE>
+  __device__ __forceinline__ static void tier(const float* src_row, float* dst_row, const float2 (&src)[Q],
+                                              float2 (&dst)[Q], int j, int M, int lo, int hi, const K& k) {
+    const int T2 = 2 * (int)blockDim.x;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int jq = j + q * T2;
+      if (jq + (ODD ? 1 : 0) < lo || jq >= hi) continue;
+      float v[2 * R + 2];
+      if constexpr (R == 2) {
+        const float2 l = *reinterpret_cast<const float2*>(src_row + jq - 2);
+        const float2 r = *reinterpret_cast<const float2*>(src_row + jq + 2);
+        v[0] = l.x, v[1] = l.y, v[4] = r.x, v[5] = r.y;
+      } else {
+        v[0] = src_row[max(jq - 1, 0)], v[3] = src_row[min(jq + 2, M - 1)];
+      }
+      v[R] = src[q].x, v[R + 1] = src[q].y;
+      const float x = Op::template point_fp<STAGE>(&v[0], dst[q].x, k);
+      const float y = Op::template point_fp<STAGE>(&v[1], dst[q].y, k);
+      if (!ODD || jq >= lo) dst[q].x = x;
+      if (!ODD || jq + 1 < hi) dst[q].y = y;
+      *reinterpret_cast<float2*>(dst_row + jq) = dst[q];
+    }
+    __syncthreads();
+  }
+  // tiers 1..n, tier s on [lo0 + d s, hi0 - d s)
+  __device__ __forceinline__ static void run(float* sm, int M, int n, int lo0, int hi0, int d, const K& k) {
+    float* row0 = sm;
+    float* row1 = sm + M;
+    const int j = J0 + 2 * (int)threadIdx.x, T2 = 2 * (int)blockDim.x;
+    float2 a[Q], b[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int jq = min(j + q * T2, M - 2);  // a pair past the window is never in a range
+      a[q] = *reinterpret_cast<const float2*>(row0 + jq);
+      b[q] = *reinterpret_cast<const float2*>(row1 + jq);
+    }
+    int lo = lo0, hi = hi0, s = 1;
+    for (; s + 1 <= n; s += 2) {
+      lo += d, hi -= d;
+      tier<0>(row0, row1, a, b, j, M, lo, hi, k);
+      lo += d, hi -= d;
+      tier<Op::S == 1 ? 0 : 1>(row1, row0, b, a, j, M, lo, hi, k);
+    }
+    if (s <= n) tier<0>(row0, row1, a, b, j, M, lo + d, hi - d, k);
+  }
+};
+// False, with nothing done, when a thread would own more than MAXQ pairs: 4, or
+// 2 out of line (with 4 there, tile 1024 and 128 threads took 1.01 ms where
+// one pair a trip takes 0.96; 8 pairs take 32 registers for the rows alone and
+// lost a third).  ODD: a range may start or end inside a pair (heat; KS with an
+// odd-sized wide tile).
+template <class Op, int MAXQ>
+__device__ __forceinline__ bool fixed_tiers(float* sm, int M, int n, int lo0, int hi0, int d,
+                                            const typename Op::K& k) {
+  const int sw = d > 0 ? 1 : n;  // the widest tier
+  if (!dbg::level(M, lo0 + d * sw, max(hi0 - d * sw, lo0 + d * sw), Op::R)) return true;
+  const int T = (int)blockDim.x, pairs = (M - 2 * (Op::R & ~1) + 1) / 2, need = (pairs + T - 1) / T;
+  if ((M & 1) || need > MAXQ) return false;
+  if (Op::R == 1 || ((lo0 | hi0) & 1)) {
+    if (need <= 1)
+      FixedTiers<Op, 1, true>::run(sm, M, n, lo0, hi0, d, k);
+    else if (need <= 2)
+      FixedTiers<Op, 2, true>::run(sm, M, n, lo0, hi0, d, k);
+    else if constexpr (MAXQ > 2)
+      FixedTiers<Op, 4, true>::run(sm, M, n, lo0, hi0, d, k);
+  } else if constexpr (Op::R == 2) {
+    if (need <= 1)
+      FixedTiers<Op, 1, false>::run(sm, M, n, lo0, hi0, d, k);
+    else if (need <= 2)
+      FixedTiers<Op, 2, false>::run(sm, M, n, lo0, hi0, d, k);
+    else if constexpr (MAXQ > 2)
+      FixedTiers<Op, 4, false>::run(sm, M, n, lo0, hi0, d, k);
+  }
+  return true;
+}
+// The same out of line, on the block's window at the start of its dynamic
+// shared memory, for the persistent and cluster kernels: inlined into their
+// many phases it spilled (KS 2^20, tile 1024, 128 threads, persistent, 500 steps: 1.81
+// ms, start 0.96).
+template <class Op>
+__device__ __noinline__ bool fixed_tiers_call(int M, int n, int lo0, int hi0, int d, typename Op::K k) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  return fixed_tiers<Op, 2>(reinterpret_cast<float*>(smraw), M, n, lo0, hi0, d, k);
+}
+
+// ---------------------------------------------------------------------------
 // device execution context for the pass phases (swept_phases.cuh)
 // ---------------------------------------------------------------------------
 // Tape: every value a pass computes at absolute tier L is also stored at
@@ -388,6 +494,7 @@ struct DevCtx {
   using value_type = T;
   using op_type = Op;
   static constexpr int kR = Op::R, kC = Op::C;
+  static constexpr bool kFixedTiers = !TAPE && sizeof(T) == 4 && Op::C == 1;
   T* sm;
   Geom g;
   typename Op::K k;
@@ -414,6 +521,10 @@ struct DevCtx {
   }
   __device__ __forceinline__ void store_edge(int r, int c, int j, int64_t e) {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e, edge_slots(g) * g.E, dbg::EDGE)) e_out[e] = row(r, c)[j];
+  }
+  // FP32: all tiers of a phase with a fixed mapping of points to threads
+  __device__ __forceinline__ bool phase_tiers(int n, int lo0, int hi0, int d, int wall) {
+    return wall == NO_WALL && fixed_tiers<Op, 4>(sm, g.M, n, lo0, hi0, d, k);
   }
   __device__ __forceinline__ void level(int s, int base, int lo, int hi, int64_t origin, int wall) {
     if (dbg::level(g.M, lo, hi, kR)) LevelImpl<T, Op>::run(sm, g.M, stage_c<Op>(s), s & 1, lo, hi, wall, g.chunk, k);
@@ -454,6 +565,7 @@ struct RegCtx : Base {
   using Op = typename Base::op_type;
   static constexpr int R = Op::R;
   static_assert(Op::C == 1 && P >= 1, "register tiers need a scalar scheme");
+  static constexpr bool kFixedTiers = false;  // its own level() keeps the whole pass in registers
   T a[P], b[P];            // rows 0 (even tiers) and 1 (odd tiers)
   T ha[2 * R], hb[2 * R];  // halo of rows 0 / 1: [0, R) -> points 0..R-1, [R, 2R) -> points W+R..W+2R-1
   bool in_regs;
@@ -584,7 +696,15 @@ __device__ __forceinline__ typename WithTiers<Base, P>::type tiers_ctx(const Bas
 // thread at 64 registers; MAXT = 256 (the variant blocks of up to 256 threads
 // run) at 85 with 3 blocks per SM, which measured faster on the Euler
 // workloads than 2 blocks of up to 128 registers.
-#define SWEPT_BOUNDS(P, MAXT) __launch_bounds__((P) > 0 ? 32 : (MAXT), (P) > 0 ? 16 : ((MAXT) <= 256 ? 3 : 1))
+// BLOCKS: of up to 256 threads per SM.  The per-pass FP32 KS kernels: 64
+// registers and 4 blocks (2^20 points, tile 1024, 128 threads,
+// 5,000 steps: 7.44 ms; with 3, 5 and 6 blocks 8.56, 8.22 and 8.96).
+template <typename T, class Op>
+constexpr int small_blocks() {
+  return sizeof(T) == 4 && Op::C == 1 && Op::R == 2 ? 4 : 3;
+}
+#define SWEPT_BOUNDS(P, MAXT, BLOCKS) \
+  __launch_bounds__((P) > 0 ? 32 : (MAXT), (P) > 0 ? 16 : ((MAXT) <= 256 ? (BLOCKS) : 1))
 
 // ---------------------------------------------------------------------------
 // persistent single-problem swept kernel: the launch sequence of
@@ -609,6 +729,7 @@ struct PDevCtx {
   using value_type = T;
   using op_type = Op;
   static constexpr int kR = Op::R, kC = Op::C;
+  static constexpr bool kFixedTiers = sizeof(T) == 4 && Op::C == 1;
   T* sm;
   Geom g;
   typename Op::K k;
@@ -634,6 +755,10 @@ struct PDevCtx {
   __device__ __forceinline__ void store_edge(int r, int c, int j, int64_t e) {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e, edge_slots(g) * g.E, dbg::EDGE)) e_out[e] = row(r, c)[j];
   }
+  // FP32: all tiers of a phase with a fixed mapping of points to threads
+  __device__ __forceinline__ bool phase_tiers(int n, int lo0, int hi0, int d, int wall) {
+    return wall == NO_WALL && fixed_tiers_call<Op>(g.M, n, lo0, hi0, d, k);
+  }
   __device__ __forceinline__ void level(int s, int, int lo, int hi, int64_t, int wall) {
     if (dbg::level(g.M, lo, hi, kR)) LevelImpl<T, Op>::run(sm, g.M, stage_c<Op>(s), s & 1, lo, hi, wall, g.chunk, k);
     __syncthreads();
@@ -651,7 +776,7 @@ __device__ __forceinline__ bool persist_wait(const int* flag, int need, const Pe
 }
 
 template <typename T, class Op, int P = 0, int MAXT = 1024>
-__global__ void SWEPT_BOUNDS(P, MAXT) k_swept_persist(Geom g, typename Op::K k, T* u, T* e0, T* e1, int64_t n_sub,
+__global__ void SWEPT_BOUNDS(P, MAXT, 3) k_swept_persist(Geom g, typename Op::K k, T* u, T* e0, T* e1, int64_t n_sub,
                                                         PersistCtl ctl) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int64_t s_item;
@@ -718,6 +843,7 @@ struct ClusterCtx {
   using value_type = T;
   using op_type = Op;
   static constexpr int kR = Op::R, kC = Op::C;
+  static constexpr bool kFixedTiers = sizeof(T) == 4 && Op::C == 1;
   T* sm;         // the block's window rows (and Euler scratch)
   T* ex_in;      // export area of the previous pass (read remotely)
   T* ex_out;     // export area this pass writes (own tile's edges)
@@ -747,6 +873,10 @@ struct ClusterCtx {
   __device__ __forceinline__ void store_edge(int r, int c, int j, int64_t e) {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e - (int64_t)my_rank * g.E, g.E, dbg::EDGE))
       ex_out[e - (int64_t)my_rank * g.E] = row(r, c)[j];
+  }
+  // FP32: all tiers of a phase with a fixed mapping of points to threads
+  __device__ __forceinline__ bool phase_tiers(int n, int lo0, int hi0, int d, int wall) {
+    return wall == NO_WALL && fixed_tiers_call<Op>(g.M, n, lo0, hi0, d, k);
   }
   __device__ __forceinline__ void level(int s, int, int lo, int hi, int64_t, int wall) {
     if (dbg::level(g.M, lo, hi, kR)) LevelImpl<T, Op>::run(sm, g.M, stage_c<Op>(s), s & 1, lo, hi, wall, g.chunk, k);
@@ -793,7 +923,7 @@ static __global__ void k_latch_error(const int* err, int* status) {
 }
 
 template <typename T, class Op, int P = 0, int MAXT = 1024>
-__global__ void SWEPT_BOUNDS(P, MAXT) k_swept_up(Geom g, typename Op::K k, const T* u_in, T* u_out, T* e_out,
+__global__ void SWEPT_BOUNDS(P, MAXT, (small_blocks<T, Op>())) k_swept_up(Geom g, typename Op::K k, const T* u_in, T* u_out, T* e_out,
                                                    int hh, int write_top) {
   extern __shared__ __align__(16) unsigned char smraw[];
   auto cx = tiers_ctx<P>(DevCtx<T, Op>{reinterpret_cast<T*>(smraw), g, k, u_in, u_out, nullptr, e_out, Tape<T>{}});
@@ -801,7 +931,7 @@ __global__ void SWEPT_BOUNDS(P, MAXT) k_swept_up(Geom g, typename Op::K k, const
 }
 
 template <typename T, class Op, int P = 0, int MAXT = 1024>
-__global__ void SWEPT_BOUNDS(P, MAXT) k_swept_diamond(Geom g, typename Op::K k, T* u_out, const T* e_in, T* e_out,
+__global__ void SWEPT_BOUNDS(P, MAXT, (small_blocks<T, Op>())) k_swept_diamond(Geom g, typename Op::K k, T* u_out, const T* e_in, T* e_out,
                                                         int odd, int mode, int hh) {
   extern __shared__ __align__(16) unsigned char smraw[];
   auto cx = tiers_ctx<P>(DevCtx<T, Op>{reinterpret_cast<T*>(smraw), g, k, nullptr, u_out, e_in, e_out, Tape<T>{}});
@@ -839,7 +969,7 @@ struct SlabCtx : DevCtx<T, Op> {
 };
 
 template <typename T, class Op, int P = 0>
-__global__ void SWEPT_BOUNDS(P, 1024) k_slab_up(Geom g, Slab sl, typename Op::K k, const T* u_in, T* u_out, T* e_out,
+__global__ void SWEPT_BOUNDS(P, 1024, 1) k_slab_up(Geom g, Slab sl, typename Op::K k, const T* u_in, T* u_out, T* e_out,
                                                 int hh, int write_top) {
   extern __shared__ __align__(16) unsigned char smraw[];
   auto cx = tiers_ctx<P>(
@@ -848,7 +978,7 @@ __global__ void SWEPT_BOUNDS(P, 1024) k_slab_up(Geom g, Slab sl, typename Op::K 
 }
 
 template <typename T, class Op, int P = 0>
-__global__ void SWEPT_BOUNDS(P, 1024) k_slab_diamond(Geom g, Slab sl, typename Op::K k, T* u_out, const T* e_in,
+__global__ void SWEPT_BOUNDS(P, 1024, 1) k_slab_diamond(Geom g, Slab sl, typename Op::K k, T* u_out, const T* e_in,
                                                      T* e_out, int odd, int mode, int hh) {
   extern __shared__ __align__(16) unsigned char smraw[];
   auto cx = tiers_ctx<P>(
