@@ -256,5 +256,32 @@ SWFIX bool square(double x, double& out) {
   return (uint32_t)(e - 600) <= 800u;
 }
 
+// 0.5 x, the same bits as the product: one off the exponent field; a subnormal
+// result shifts the magnitude, ties to even; zeros, infinities and NaN stay
+SWFIX double half(double x) {
+  const uint32_t hi = dhi(x), lo = dlo(x), e = hi & 0x7ff00000u;
+  const bool normal = e - 0x00200000u < 0x7fd00000u;
+  uint32_t h = hi - (normal ? 0x00100000u : 0u), l = lo;
+  if (e < 0x00200000u && ((hi << 1) | lo) != 0u) {
+    const uint64_t m = ((uint64_t)(hi & 0x7fffffffu) << 32) | lo, r = (m + ((m >> 1) & 1u)) >> 1;
+    h = (hi & 0x80000000u) | (uint32_t)(r >> 32);
+    l = (uint32_t)r;
+  }
+  return make_double(h, l);
+}
+// x positive and within 2^-60 .. 2^59
+SWFIX bool mid(double x) { return dhi(x) - (963u << 20) < (120u << 20); }
+// x truncated to a float, for 2^-126 <= |x| < 2^128
+SWFIX float float_bits(double x) {
+  const uint32_t hi = dhi(x), b = (hi & 0x80000000u) | (((hi & 0x7fffffffu) - 0x38000000u) << 3) | (dlo(x) >> 29);
+#if defined(__CUDA_ARCH__)
+  return __uint_as_float(b);
+#else
+  float f;
+  memcpy(&f, &b, 4);
+  return f;
+#endif
+}
+
 }  // namespace fix
 }  // namespace swept

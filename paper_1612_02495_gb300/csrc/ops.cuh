@@ -153,6 +153,10 @@ __device__ __forceinline__ double max_nonneg(double a, double b) {
 }
 __device__ __forceinline__ float max_nonneg(float a, float b) { return __float_as_int(a) >= __float_as_int(b) ? a : b; }
 
+// 0.5 x, in FP64 on the integer pipe
+__device__ __forceinline__ float half_of(float x) { return mul_rn(0.5f, x); }
+__device__ __forceinline__ double half_of(double x) { return fix::half(x); }
+
 template <typename T>
 struct EulerOp {
   static constexpr int R = 2, S = 2, C = 3;
@@ -166,7 +170,7 @@ struct EulerOp {
     Prim w;
     w.r = r;
     w.u = div_rn(m, r);
-    w.p = mul_rn(k.gm1, fma_rn(-mul_rn(T(0.5), m), w.u, e));
+    w.p = mul_rn(k.gm1, fma_rn(-half_of(m), w.u, e));
     return w;
   }
   // One side of a face: the MUSCL-minmod reconstructed state with its
@@ -175,48 +179,85 @@ struct EulerOp {
   struct Side {
     T r, u, p, m, E, sp;
   };
-  __device__ __forceinline__ static void finish_side(Side& X, const K& k) {
+  __device__ __forceinline__ static T speed(T r, T u, T p, T gamma) {
+    return add_rn(fabs(u), sqrt_rn(div_rn(mul_rn(gamma, p), r)));
+  }
+  __device__ __noinline__ static T speed_cold(T r, T u, T p, T gamma) { return speed(r, u, p, gamma); }
+  __device__ __forceinline__ static void finish_state(Side& X, const K& k) {
     X.m = mul_rn(X.r, X.u);
-    X.E = fma_rn(mul_rn(T(0.5), X.m), X.u, mul_rn(X.p, k.igm1));
-    const T c = sqrt_rn(div_rn(mul_rn(k.gamma, X.p), X.r));
-    X.sp = add_rn(fabs(X.u), c);
+    X.E = fma_rn(half_of(X.m), X.u, mul_rn(X.p, k.igm1));
   }
-  __device__ __forceinline__ static Side left_side(const Prim& a, const Prim& b, const Prim& c, const K& k) {
-    Side L;
-    L.r = add_rn(b.r, mul_rn(T(0.5), minmod(sub_rn(b.r, a.r), sub_rn(c.r, b.r))));
-    L.u = add_rn(b.u, mul_rn(T(0.5), minmod(sub_rn(b.u, a.u), sub_rn(c.u, b.u))));
-    L.p = add_rn(b.p, mul_rn(T(0.5), minmod(sub_rn(b.p, a.p), sub_rn(c.p, b.p))));
-    finish_side(L, k);
-    return L;
+  __device__ __forceinline__ static void finish_side(Side& X, const K& k) {
+    finish_state(X, k);
+    X.sp = speed(X.r, X.u, X.p, k.gamma);
   }
-  __device__ __forceinline__ static Side right_side(const Prim& b, const Prim& c, const Prim& d, const K& k) {
-    Side R;
-    R.r = sub_rn(c.r, mul_rn(T(0.5), minmod(sub_rn(c.r, b.r), sub_rn(d.r, c.r))));
-    R.u = sub_rn(c.u, mul_rn(T(0.5), minmod(sub_rn(c.u, b.u), sub_rn(d.u, c.u))));
-    R.p = sub_rn(c.p, mul_rn(T(0.5), minmod(sub_rn(c.p, b.p), sub_rn(d.p, c.p))));
-    finish_side(R, k);
-    return R;
+  // the reconstructed states, without momentum, energy and speed
+  __device__ __forceinline__ static void left_state(Side& L, const Prim& a, const Prim& b, const Prim& c) {
+    L.r = add_rn(b.r, half_of(minmod(sub_rn(b.r, a.r), sub_rn(c.r, b.r))));
+    L.u = add_rn(b.u, half_of(minmod(sub_rn(b.u, a.u), sub_rn(c.u, b.u))));
+    L.p = add_rn(b.p, half_of(minmod(sub_rn(b.p, a.p), sub_rn(c.p, b.p))));
+  }
+  __device__ __forceinline__ static void right_state(Side& R, const Prim& b, const Prim& c, const Prim& d) {
+    R.r = sub_rn(c.r, half_of(minmod(sub_rn(c.r, b.r), sub_rn(d.r, c.r))));
+    R.u = sub_rn(c.u, half_of(minmod(sub_rn(c.u, b.u), sub_rn(d.u, c.u))));
+    R.p = sub_rn(c.p, half_of(minmod(sub_rn(c.p, b.p), sub_rn(d.p, c.p))));
   }
   // Rusanov flux from the two sides: 1/2 (F(L) + F(R)) - 1/2 s (U_R - U_L),
   // s = the larger of |u| + c over the two sides
   // sp = |u| + c >= 0 on both sides
   __device__ __forceinline__ static T smax(const Side& L, const Side& R) { return max_nonneg(L.sp, R.sp); }
+  // The same, from the states alone.  A division and a square root are 26 of the
+  // 127 FP64 pipe slots a cell and sub-step took with both sides' speeds, so in
+  // FP64 only the faster side's is computed: which it is shows in single
+  // precision (from truncated bits, no FP64 instruction) when the estimates differ
+  // by more than 2^-20 of their sum.  An estimate is within 2^-21.3 of its speed:
+  // truncated p, rho and gamma, the product and the quotient give 2^-21.2, halved
+  // by the root; the root, truncated |u| and the sum 2^-23, 2^-23 and 2^-24.
+  // Sides with the same bits have the same speed; everything else computes both.
+  __device__ __forceinline__ static T speed_max(const Side& L, const Side& R, const K& k) {
+    if constexpr (sizeof(T) == 8) {
+      const uint32_t ml = fix::mag(L.u), mr = fix::mag(R.u);
+      const float g = fix::float_bits(k.gamma);
+      const float ul = ml < (923u << 20) ? 0.f : fabsf(fix::float_bits(L.u));  // below 2^-100: nothing beside c
+      const float ur = mr < (923u << 20) ? 0.f : fabsf(fix::float_bits(R.u));
+      float cl, cr;
+      asm("sqrt.approx.f32 %0, %1;" : "=f"(cl) : "f"(__fdividef(g * fix::float_bits(L.p), fix::float_bits(L.r))));
+      asm("sqrt.approx.f32 %0, %1;" : "=f"(cr) : "f"(__fdividef(g * fix::float_bits(R.p), fix::float_bits(R.r))));
+      const float sl = ul + cl, sr = ur + cr;
+      const bool left = sl > sr;
+      // p, rho and gamma within 2^-60 .. 2^59 (positive), |u| below 2^60
+      const bool fits = fix::mid(L.p) && fix::mid(L.r) && fix::mid(R.p) && fix::mid(R.r) && fix::mid(k.gamma) &&
+                        fix::umax(ml, mr) < (1083u << 20);
+      const bool same = __double_as_longlong(L.p) == __double_as_longlong(R.p) &&
+                        __double_as_longlong(L.r) == __double_as_longlong(R.r) &&
+                        __double_as_longlong(L.u) == __double_as_longlong(R.u);
+      T s = speed(left ? L.r : R.r, left ? L.u : R.u, left ? L.p : R.p, k.gamma);
+      if (!((fits && fabsf(sl - sr) > (sl + sr) * 0x1p-20f) || same))
+        s = max_nonneg(s, speed_cold(left ? R.r : L.r, left ? R.u : L.u, left ? R.p : L.p, k.gamma));
+      return s;
+    } else {
+      return max_nonneg(speed(L.r, L.u, L.p, k.gamma), speed(R.r, R.u, R.p, k.gamma));
+    }
+  }
   __device__ __forceinline__ static T flux0(const Side& L, const Side& R, T s) {
-    return mul_rn(T(0.5), fma_rn(-s, sub_rn(R.r, L.r), add_rn(L.m, R.m)));
+    return half_of(fma_rn(-s, sub_rn(R.r, L.r), add_rn(L.m, R.m)));
   }
   __device__ __forceinline__ static T flux1(const Side& L, const Side& R, T s) {
-    return mul_rn(T(0.5), fma_rn(-s, sub_rn(R.m, L.m), add_rn(fma_rn(L.m, L.u, L.p), fma_rn(R.m, R.u, R.p))));
+    return half_of(fma_rn(-s, sub_rn(R.m, L.m), add_rn(fma_rn(L.m, L.u, L.p), fma_rn(R.m, R.u, R.p))));
   }
   __device__ __forceinline__ static T flux2(const Side& L, const Side& R, T s) {
-    return mul_rn(T(0.5),
-                  fma_rn(-s, sub_rn(R.E, L.E), add_rn(mul_rn(L.u, add_rn(L.E, L.p)), mul_rn(R.u, add_rn(R.E, R.p)))));
+    return half_of(
+        fma_rn(-s, sub_rn(R.E, L.E), add_rn(mul_rn(L.u, add_rn(L.E, L.p)), mul_rn(R.u, add_rn(R.E, R.p)))));
   }
   // Rusanov flux through the face between cells b and c, from cells a, b, c, d
   __device__ __forceinline__ static void flux(const Prim& a, const Prim& b, const Prim& c, const Prim& d, const K& k,
                                               T& F0, T& F1, T& F2) {
-    const Side L = left_side(a, b, c, k);
-    const Side R = right_side(b, c, d, k);
-    const T s = smax(L, R);
+    Side L, R;
+    left_state(L, a, b, c);
+    right_state(R, b, c, d);
+    const T s = speed_max(L, R, k);
+    finish_state(L, k);
+    finish_state(R, k);
     F0 = flux0(L, R, s);
     F1 = flux1(L, R, s);
     F2 = flux2(L, R, s);
@@ -225,7 +266,7 @@ struct EulerOp {
   __device__ __forceinline__ static T update(T fp, T fm, T in_self, T prev2, const K& k) {
     if (STAGE == 0) return fma_rn(k.mdtdx, sub_rn(fp, fm), in_self);
     const T t = fma_rn(k.mdtdx, sub_rn(fp, fm), in_self);
-    return mul_rn(T(0.5), add_rn(prev2, t));
+    return half_of(add_rn(prev2, t));
   }
 };
 

@@ -44,6 +44,16 @@ int main(int argc, char** argv) {
       wrong += bits(d4) != bits(std::fma(6.0, v[2], std::fma(-4.0, s1, s2)));
     }
     if (square(v[0], q)) wrong += bits(q) != bits(v[0] * v[0]);
+    // half: any bit pattern, and the smallest exponents
+    uint64_t p = g();
+    if (it & 1) p &= 0x803fffffffffffffull;
+    double h;
+    memcpy(&h, &p, 8);
+    if (h == h) wrong += bits(half(h)) != bits(0.5 * h);
+    if (std::fabs(h) > 1e-37 && std::fabs(h) < 1e38)
+      wrong += std::fabs((double)float_bits(h) - h) > 0x1p-23 * std::fabs(h) || std::fabs((double)float_bits(h)) > std::fabs(h);
+    const float fb = float_bits(v[1]);
+    wrong += !(std::fabs((double)fb) <= std::fabs(v[1]) && std::fabs((double)fb - v[1]) <= 0x1p-23 * std::fabs(v[1])) && kind != 8;
     // a value outside the range in any place is refused
     const double out[5] = {0.0, -0.0, 1e-310, std::numeric_limits<double>::infinity(), std::nan("")};
     v[g() % 5] = out[g() % 5];
