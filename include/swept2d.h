@@ -47,7 +47,11 @@ extern "C" {
  *   tile_w   W: the tile is W x W points, W a multiple of 4 (so that the half
  *            cycle h = W / 2 is even), 8 <= W <= 64 for FP64 and <= 128 for
  *            FP32 (two (W + 2)^2 level rows in shared memory); 0 = library choice
- *   threads  threads per block, a multiple of 32, <= 1024; 0 = 256
+ *   threads  threads per block, a multiple of 32, <= 1024; 0 = 256.  With tile_w,
+ *            threads and persistent all 0 the library also chooses the
+ *            decomposition: swept2d_step_n advances overlapped tiles (each with a
+ *            frame of ghost points, a few steps a launch) through the second
+ *            array of the workspace; the values are the same bit for bit
  *   persistent  0: one launch per pass (pyramid, then a bridge launch and an
  *            octahedron launch per half cycle); 1: one persistent launch whose
  *            resident blocks run the same pieces from a queue in launch order,

@@ -227,6 +227,36 @@ SWFIX bool second_fourth(double a, double b, double c, double d, double e, doubl
   return ok;
 }
 
+// Neighbour sums of a run of L points v of one column, with the points above and
+// below the run and the rows' neighbours w[i ST], e[i ST] (ST their stride):
+//   s[i] = (w_i + e_i) + (v_{i-1} + v_{i+1}), each sum correctly rounded.
+// One scale for the run, so a column value is converted once for the two sums it is
+// in.  False (s meaningless) when any value is outside the range.
+template <int L, int ST>
+SWFIX bool cross_sums(const double* w, const double* e, double up, double down, const double (&v)[L],
+                      double (&s)[L]) {
+  uint32_t lo = umin(mag(up), mag(down)), hi = umax(mag(up), mag(down));
+#pragma unroll
+  for (int i = 0; i < L; ++i) {
+    const uint32_t a = mag(v[i]), b = mag(w[i * ST]), c = mag(e[i * ST]);
+    lo = umin(lo, umin(a, umin(b, c)));
+    hi = umax(hi, umax(a, umax(b, c)));
+  }
+  int E;
+  bool ok = in_range(lo, hi, E);
+  const int sh0 = kG - E;
+  F96 below = load(up, sh0), own = load(v[0], sh0);
+#pragma unroll
+  for (int i = 0; i < L; ++i) {
+    const F96 above = load(i + 1 < L ? v[i + 1] : down, sh0);
+    const F96 sx = round53(add(load(w[i * ST], sh0), load(e[i * ST], sh0)));
+    s[i] = to_double(add(sx, round53(add(below, above))), E, ok);
+    below = own;
+    own = above;
+  }
+  return ok;
+}
+
 // x * x, correctly rounded; false outside the range
 SWFIX bool square(double x, double& out) {
   const uint32_t w = mag(x), ml = dlo(x), mh = (w & 0xfffffu) | 0x100000u;

@@ -44,6 +44,14 @@ int main(int argc, char** argv) {
       wrong += bits(d4) != bits(std::fma(6.0, v[2], std::fma(-4.0, s1, s2)));
     }
     if (square(v[0], q)) wrong += bits(q) != bits(v[0] * v[0]);
+    if (it % 8 == 0) {  // a column run of four points, rows of stride 3: (w, own, e)
+      double a[12], col[4], sum[4];
+      for (int i = 0; i < 12; ++i) a[i] = v[g() % 5] * (1.0 + (double)(g() >> 40) * 0x1p-26);
+      for (int i = 0; i < 4; ++i) col[i] = a[3 * i + 1];
+      if (cross_sums<4, 3>(a, a + 2, v[0], v[4], col, sum))
+        for (int i = 0; i < 4; ++i)
+          wrong += bits(sum[i]) != bits((a[3 * i] + a[3 * i + 2]) + ((i ? col[i - 1] : v[0]) + (i < 3 ? col[i + 1] : v[4])));
+    }
     // half: any bit pattern, and the smallest exponents
     uint64_t p = g();
     if (it & 1) p &= 0x803fffffffffffffull;
