@@ -212,13 +212,17 @@ SWFIX bool in_range(uint32_t lo_mag, uint32_t hi_mag, int& E) {
 // The linear part of a five-point fourth-order stencil:
 //   sp1 = d + b;  sp2 = e + a;  d2 = fma(-2, c, sp1);  d4 = fma(6, c, fma(-4, sp1, sp2))
 // each correctly rounded.  False (d2, d4 meaningless) outside the range.
-SWFIX bool second_fourth(double a, double b, double c, double d, double e, double& d2, double& d4) {
+// With `bd`, also *bd = b - d.
+SWFIX bool second_fourth(double a, double b, double c, double d, double e, double& d2, double& d4,
+                         double* bd = nullptr) {
   const uint32_t wa = mag(a), wb = mag(b), wc = mag(c), wd = mag(d), we = mag(e);
   int E;
   bool ok = in_range(umin(umin(umin(wa, wb), umin(wd, we)), wc), umax(umax(umax(wa, wb), umax(wd, we)), wc), E);
   const int sh0 = kG - E;
-  const F96 s1 = round53(add(load(d, sh0), load(b, sh0)));
+  const F96 xb = load(b, sh0), xd = load(d, sh0);
+  const F96 s1 = round53(add(xd, xb));
   const F96 s2 = round53(add(load(e, sh0), load(a, sh0)));
+  if (bd) *bd = to_double(sub(xb, xd), E, ok);
   const F96 c1 = load(c, sh0), c2 = add(c1, c1);
   d2 = to_double(sub(s1, c2), E, ok);
   const F96 t1 = add(s1, s1);

@@ -535,7 +535,7 @@ struct DevCtx {
       const int64_t slot = tape.base + base + s - tape.tier0;
       if (slot >= 0 && slot < tape.ntiers)
         for (int j = lo + (int)threadIdx.x; j < hi; j += (int)blockDim.x) {
-          const int64_t x = wrap_n(origin + j, g.N);
+          const int64_t x = wrap_near(origin + j, g.N);
 #pragma unroll
           for (int c = 0; c < Op::C; ++c) tape.p[(slot * Op::C + c) * g.N + x] = row(s & 1, c)[j];
         }
@@ -1021,11 +1021,54 @@ __device__ __forceinline__ void adjoint_level(T* sm, int M, int stage, int out_r
     T v[2 * R + 1];
 #pragma unroll
     for (int d = 0; d <= 2 * R; ++d) v[d] = in[nbr(j, d - R, wall)];
-    const T w = fwd[wrap_n(origin + j, N)];
+    const T w = fwd[wrap_near(origin + j, N)];
     if (stage == 0)
       out[j] = AOp::template point<0>(v, T(0), w, k, acc);
     else
       out[j] = AOp::template point<1>(v, out[j], w, k, acc);
+  }
+}
+
+// The KS adjoint in FP64: as ks_f64_level, with the forward state of the tier
+// (`fwd`, global memory) and the parameter's sum.  `ahead`: the next tier's
+// forward state, asked into L1 now, because a tier is shorter than a read from L2.
+template <int STAGE>
+__device__ __noinline__ void ks_adj_redo(const double* in, double* out, int lo, int hi, int64_t origin, int64_t N,
+                                         const double* fwd, KsAdjOp<double>::K k, KahanAcc* acc) {
+  using A = KsAdjOp<double>;
+  KahanAcc a = *acc;
+  for (int j = lo + (int)threadIdx.x; j < hi; j += (int)blockDim.x) {
+    KahanAcc none;
+    double r;
+    const double p2 = STAGE == 1 ? out[j] : 0.0, w = fwd[wrap_near(origin + j, N)];
+    if (!A::point_int<STAGE>(in + j - 2, p2, w, k, none, r)) out[j] = A::point<STAGE>(in + j - 2, p2, w, k, a);
+  }
+  *acc = a;
+}
+template <int STAGE>
+__device__ __forceinline__ void ks_adj_level(double* sm, int M, int out_row, int lo, int hi, int64_t origin, int64_t N,
+                                             const double* fwd, const double* ahead, const KsAdjOp<double>::K& k,
+                                             KahanAcc& acc) {
+  const double* in = sm + (out_row ^ 1) * M;
+  double* out = sm + out_row * M;
+  bool bad = false;
+  for (int j = lo + (int)threadIdx.x; j < hi; j += (int)blockDim.x) {
+    double v[5];
+#pragma unroll
+    for (int d = 0; d < 5; ++d) v[d] = in[j + d - 2];
+    const int64_t x = wrap_near(origin + j, N);
+    const double w = fwd[x];
+    if (ahead) asm volatile("prefetch.global.L1 [%0];" ::"l"(ahead + x));
+    const double p2 = STAGE == 1 ? out[j] : 0.0;
+    double r;
+    const bool ok = KsAdjOp<double>::point_int<STAGE>(v, p2, w, k, acc, r);
+    if (ok) out[j] = r;
+    bad = bad || !ok;
+  }
+  if (bad) {
+    KahanAcc a = acc;
+    ks_adj_redo<STAGE>(in, out, lo, hi, origin, N, fwd, k, &a);
+    acc = a;
   }
 }
 
@@ -1065,7 +1108,15 @@ struct AdjCtx {
   __device__ __forceinline__ void level(int s, int b, int lo, int hi, int64_t origin, int wall) {
     const int64_t L = base + b + s;
     if (dbg::level(g.M, lo, hi, kR) && dbg::ok(top - L >= 0 && top - L <= top, dbg::TAPE, L))
-      adjoint_level<T, AOp>(sm, g.M, stage_c<AOp>(s), s & 1, lo, hi, wall, origin, g.N, tape + (top - L) * g.N, k,
+      if constexpr (std::is_same<AOp, KsAdjOp<double>>::value) {
+        const double* fwd = tape + (top - L) * g.N;
+        const double* ahead = top - L > 0 ? fwd - g.N : nullptr;
+        if (s & 1)
+          ks_adj_level<0>(sm, g.M, s & 1, lo, hi, origin, g.N, fwd, ahead, k, acc);
+        else
+          ks_adj_level<1>(sm, g.M, s & 1, lo, hi, origin, g.N, fwd, ahead, k, acc);
+      } else
+        adjoint_level<T, AOp>(sm, g.M, stage_c<AOp>(s), s & 1, lo, hi, wall, origin, g.N, tape + (top - L) * g.N, k,
                             acc);
     __syncthreads();
   }

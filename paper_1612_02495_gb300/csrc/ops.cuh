@@ -314,6 +314,21 @@ struct KsAdjOp {
     d4 = fma_rn(T(6), v[2], fma_rn(T(-4), sp1, sp2));
     return fma_rn(k.c4, d4, fma_rn(k.c2, d2, nl));
   }
+  // FP64: the three sums and differences on the integer pipes (fixadd.cuh), 11 or
+  // 12 of the 17 or 18 operations on the FP64 pipe.  False, with nothing
+  // accumulated, where they do not handle an operand; the caller then takes point.
+  template <int STAGE>
+  __device__ __forceinline__ static bool point_int(const T* v, T prev2, T w, const K& k, KahanAcc& acc, T& r) {
+    T d2, d4, dl;
+    const bool ok = fix::second_fourth(v[0], v[1], v[2], v[3], v[4], d2, d4, &dl);
+    const T g = fma_rn(k.c4, d4, fma_rn(k.c2, d2, mul_rn(mul_rn(k.ca2, w), dl)));
+    r = STAGE == 0 ? mul_rn(k.mdt, g) : fma_rn(k.mdth, g, add_rn(prev2, v[2]));
+    KahanAcc sum = acc;
+    sum.add((double)mul_rn(mul_rn(STAGE == 0 ? k.mdtk4 : k.mdthk4, d4), w));
+    acc.s = ok ? sum.s : acc.s;
+    acc.c = ok ? sum.c : acc.c;
+    return ok;
+  }
   template <int STAGE>
   __device__ __forceinline__ static T point(const T* v, T prev2, T w, const K& k, KahanAcc& acc) {
     T d4;

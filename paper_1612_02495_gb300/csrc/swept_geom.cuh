@@ -82,6 +82,11 @@ SW_HD int64_t wrap_n(int64_t x, int64_t n) {
   return r < 0 ? r + n : r;
 }
 
+// the same for -n <= x < 2n, which holds for every point of a window (it
+// starts at most R points before 0 and ends less than a tile after n), without
+// the division: a 64-bit remainder is about 100 instructions
+SW_HD int64_t wrap_near(int64_t x, int64_t n) { return x < 0 ? x + n : (x >= n ? x - n : x); }
+
 // stage (0-based) of the update that produces sub-timestep level s >= 1
 SW_HD int stage_of(const Geom& g, int s) { return (s - 1) % g.S; }
 

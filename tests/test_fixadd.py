@@ -37,6 +37,8 @@ int main(int argc, char** argv) {
       for (int i = 0; i < 5; ++i) v[i] = c + (i - 2) * h + (i - 2) * (i - 2) * h * std::ldexp(1.0, -(int)(g() % 8));
     }
     double d2, d4, q;
+    double bd;
+    if (second_fourth(v[0], v[1], v[2], v[3], v[4], d2, d4, &bd)) wrong += bits(bd) != bits(v[1] - v[3]);
     if (second_fourth(v[0], v[1], v[2], v[3], v[4], d2, d4)) {
       ++handled;
       const double s1 = v[3] + v[1], s2 = v[4] + v[0];
