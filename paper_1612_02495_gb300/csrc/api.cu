@@ -51,24 +51,46 @@ const SchemeImpl* pick_impl(int scheme, int dtype) {
 bool tile_ok(int64_t n, int W, int R) { return W >= 4 * R && W % (4 * R) == 0 && n / W >= 2; }
 bool tile_divides(int64_t n, int W, int R) { return tile_ok(n, W, R) && n % W == 0; }
 
+// Narrowest default tile.  On a grid that cannot fill the GPU a pass costs its
+// launch and its 2h dependent tiers whatever their width, so wider tiles (more
+// sub-timesteps a launch) win until a tier no longer fits its block's warps.  Measured
+// microseconds a timestep, tiles that give two blocks a SM against this width:
+//   KS FP32    4096: 2.52 / 0.48   16384: 0.97 / 0.48   65536: 0.63 / 0.54
+//   KS FP64    4096: 3.45 / 1.90   16384: 2.34 / 1.93   65536: 3.18 / 3.17
+//   heat FP32  4096: 0.78 / 0.26   65536: 0.30 / 0.27
+//   heat FP64  4096: 0.97 / 0.56   65536: 0.78 / 0.76
+//   Euler FP32 4096: 4.89 / 3.19   16384: 3.64 / 3.16   65536: 3.66 / 3.61
+//   Euler FP64 16384: 23.4 / 21.9  65536: 37.5 / 35.2   (4096: 21.0 / 21.8: none below 8192)
+//   KS forward and adjoint 4096: 25.3 / 10.1   32768: 16.5 / 10.8   65536: 16.9 / 14.7
+int narrowest_tile(int64_t n, int scheme, int dtype) {
+  if (dtype == SWEPT_F32) return 256;
+  if (scheme == SWEPT_EULER) return n < 8192 ? 0 : (n < 65536 ? 128 : 256);
+  return n < 32768 ? 128 : 256;
+}
+
 // Default tile width: the largest W <= 1024 (multiple of 4R, dividing n) that
 // still gives at least two blocks per SM; else at least one per SM; else the
 // smallest such W.  When no multiple of 4R divides n, the same rules choose
 // among all legal widths (the last tile then carries the n mod W extra points).
-int choose_tile(int64_t n, int R, int sms) {
-  for (int pass = 0; pass < 2; ++pass) {
-    auto ok = [&](int W) { return pass == 0 ? tile_divides(n, W, R) : tile_ok(n, W, R); };
-    int best = 0;
-    for (int W = 4 * R; W <= 1024; W += 4 * R)
-      if (ok(W) && n / W >= 2 * sms) best = W;
-    if (best) return best;
-    for (int W = 4 * R; W <= 1024; W += 4 * R)
-      if (ok(W) && n / W >= sms) best = W;
-    if (best) return best;
-    for (int W = 4 * R; W <= 4096; W += 4 * R)
-      if (ok(W)) return W;
+// A width below `narrowest` (at most n / 2) gives way to the smallest
+// dividing width of up to twice that, or to that width itself.
+int choose_tile(int64_t n, int R, int sms, int narrowest) {
+  int W = 0;
+  for (int pass = 0; pass < 2 && !W; ++pass) {
+    auto ok = [&](int w) { return pass == 0 ? tile_divides(n, w, R) : tile_ok(n, w, R); };
+    for (int w = 4 * R; w <= 1024; w += 4 * R)
+      if (ok(w) && n / w >= 2 * sms) W = w;
+    if (W) break;
+    for (int w = 4 * R; w <= 1024; w += 4 * R)
+      if (ok(w) && n / w >= sms) W = w;
+    for (int w = 4 * R; w <= 4096 && !W; w += 4 * R)
+      if (ok(w)) W = w;
   }
-  return 0;
+  const int least = (int)std::min<int64_t>(narrowest, n / 2) / (4 * R) * (4 * R);
+  if (W == 0 || W >= least) return W;
+  for (int w = least; w <= 2 * least; w += 4 * R)
+    if (tile_divides(n, w, R)) return w;
+  return least;
 }
 
 // The resident kernel (resident.cuh) for an n-point grid, or P = 0 where the
@@ -80,17 +102,17 @@ int choose_tile(int64_t n, int R, int sms) {
 // smallest sum over points per lane, warps and blocks is taken; it came out 10
 // to 30 cycles below what was measured.  Beyond `limit` the swept passes are
 // faster.  Measured cycles per sub-timestep, resident against the default tile:
-//   heat FP32  1024: 94 / 2420   8192: 94 / 958    32768: 150 / 621
-//   heat FP64  1024: 373 / 2706  4096: 843 / 1790  8192: 1477 / 1303
-//   KS FP32    1024: 134 / 2357  8192: 175 / 1422  16384: 264 / 977  32768: 393 / 742
-//   KS FP64    1024: 1061 / 3113 4096: 2692 / 3206 8192: 4756 / 2541
+//   heat FP32  1024: 94 / 559     8192: 94 / 559     32768: 150 / 559
+//   heat FP64  1024: 373 / 1221   4096: 843 / 1159   8192: 1477 / 1300
+//   KS FP32    1024: 134 / 486    8192: 175 / 500    16384: 264 / 497  32768: 393 / 507
+//   KS FP64    1024: 1061 / 1935  2048: 1789 / 1950  4096: 2692 / 1966
 swept::ResidentPlan choose_resident(int64_t n, const SchemeImpl* im) {
   swept::ResidentPlan best;
   if (!im->resident || n > 65536) return best;
   const bool f64 = im->value_bytes == 8;
   const int ops = im->R == 1 ? 3 : 11, N = (int)n;
   const double per_op = f64 ? 64.0 : 1.0, chain = f64 ? 64.0 : (im->R == 1 ? 8.0 : 25.0);
-  const double limit = f64 ? (im->R == 1 ? 1000.0 : 2600.0) : 350.0;
+  const double limit = f64 ? (im->R == 1 ? 1000.0 : 1700.0) : 350.0;
   double best_t = limit;
   for (int P = 1; P <= 8; P *= 2)
     for (int blocks = 1; blocks <= 16; blocks *= 2)
@@ -372,7 +394,7 @@ swept_status swept_init(const swept_config* cfg, swept_handle** out) {
   cudaGetLastError();  // clear a no-device error
   cudaError_t e = cudaSuccess;
   const int R = im->R;
-  const int W = cfg->tile_w > 0 ? cfg->tile_w : choose_tile(cfg->n, R, h->sm_count);
+  const int W = cfg->tile_w > 0 ? cfg->tile_w : choose_tile(cfg->n, R, h->sm_count, narrowest_tile(cfg->n, cfg->scheme, cfg->dtype));
   // an explicit tile must be legal; with the library's choice, a grid too
   // small for two tiles of 4R points still gets a handle for classic_step_n
   if (cfg->tile_w != 0 && (cfg->tile_w < 0 || !tile_ok(cfg->n, W, R))) {
