@@ -15,7 +15,7 @@
 //                                  compute sub-timestep (base + s) on [lo, hi)
 //                                  into row s&1 from row (s-1)&1 (and row s&1
 //                                  for the second stage), then sync
-//   kFixedTiers (optional)           the context has phase_tiers (run_tiers)
+//   kFixedTiers (optional)           the context has phase_tiers (run_phase)
 //   kSlab (optional, with member `sl`)
 //                                  the context runs one slab of a grid split
 //                                  over ranks: edge indices go to the slab's
@@ -69,12 +69,14 @@ struct has_phase_tiers : std::false_type {};
 template <class Cx>
 struct has_phase_tiers<Cx, std::enable_if_t<Cx::kFixedTiers>> : std::true_type {};
 
-// tiers s = 1..n of a phase on [lo0 + d s, hi0 - d s): d = R shrinks, -R grows
+// all tiers s = 1..n of a phase on [lo0 + d s, hi0 - d s) (d = R shrinks, -R
+// grows) where the context can; false: they are still to be run, one by one
 template <class Cx>
-SW_HD void run_tiers(Cx& cx, int n, int base, int lo0, int hi0, int d, int64_t origin, int wall) {
+SW_HD bool run_phase(Cx& cx, int n, int lo0, int hi0, int d, int wall) {
   if constexpr (has_phase_tiers<Cx>::value)
-    if (cx.phase_tiers(n, lo0, hi0, d, wall)) return;
-  for_tiers(n, [&](int s) { cx.level(s, base, lo0 + d * s, hi0 - d * s, origin, wall); });
+    return cx.phase_tiers(n, lo0, hi0, d, wall);
+  else
+    return false;
 }
 
 // Up-triangle (pass 0, Fig. SweptPseudo) or, with hh < h, the trapezoid that
@@ -94,7 +96,8 @@ SW_HD void run_up(Cx& cx, const Geom& g_in, int64_t b, int hh, bool write_top) {
     cx.load_u(0, c, g.R + k, x0 + k);
   });
   cx.sync();
-  run_tiers(cx, hh, 0, g.R, g.R + w, g.R, origin, NO_WALL);
+  if (!run_phase(cx, hh, g.R, g.R + w, g.R, NO_WALL))
+    for_tiers(hh, [&](int s) { cx.level(s, 0, g.R + g.R * s, g.R + w - g.R * s, origin, NO_WALL); });
   const int per_level = g.C * 2 * g.R;
   const int per_side = hh * per_level;
   cx.for_range(0, 2 * per_side, [&](int i) {
@@ -166,10 +169,12 @@ SW_HD void run_diamond(Cx& cx, const Geom& g_in, int64_t b, int odd, int mode, i
   }
   cx.sync();
   const int wall = window_wall(g, origin, w + 2 * g.R);
-  run_tiers(cx, hh, 0, dofs + grow_lo(g, 0), dofs + grow_hi(g, 0), -g.R, origin, wall);
+  if (!run_phase(cx, hh, dofs + grow_lo(g, 0), dofs + grow_hi(g, 0), -g.R, wall))
+    for_tiers(hh, [&](int s) { cx.level(s, 0, dofs + grow_lo(g, s), dofs + grow_hi(g, s), origin, wall); });
   if (mode == MODE_DIAMOND) {
     const int top = wide ? g.h : g.h - 1;  // a triangle's tier h is empty; a wide tile's is its flat top
-    run_tiers(cx, top, g.h, g.R, g.R + w, g.R, origin, wall);
+    if (!run_phase(cx, top, g.R, g.R + w, g.R, wall))
+      for_tiers(top, [&](int s) { cx.level(s, g.h, g.R + g.R * s, g.R + w - g.R * s, origin, wall); });
     const int per_side_h = g.h * per_level;
     cx.for_range(0, 2 * per_side_h, [&](int i) {
       const int side = i >= per_side_h ? 1 : 0;
