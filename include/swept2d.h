@@ -50,8 +50,8 @@ extern "C" {
  *   threads  threads per block, a multiple of 32, <= 1024; 0 = 256.  With tile_w,
  *            threads and persistent all 0 the library also chooses the
  *            decomposition: swept2d_step_n advances overlapped tiles (each with a
- *            frame of ghost points, a few steps a launch) through the second
- *            array of the workspace; the values are the same bit for bit
+ *            frame of ghost points, a few steps a launch), u and a part of the
+ *            workspace in turn; the values are the same bit for bit
  *   persistent  0: one launch per pass (pyramid, then a bridge launch and an
  *            octahedron launch per half cycle); 1: one persistent launch whose
  *            resident blocks run the same pieces from a queue in launch order,

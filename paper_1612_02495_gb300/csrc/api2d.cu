@@ -191,7 +191,8 @@ cudaError_t issue_overlap_l(swept2d_handle* h, T* u, int64_t n, int64_t total, i
   const dim3 grid((unsigned)((g.nx + ox - 1) / ox), (unsigned)((g.ny + oy - 1) / oy));
   const size_t smem = swept2d::tile2d_smem<T>(L);
   const auto k = consts<T>(h);
-  T* tmp = (T*)(h->ws + h->off_tmp);
+  // the other array: the first strip buffer (classic2d_step_n on another stream owns off_tmp)
+  T* tmp = (T*)(h->ws + h->off_s0);
   cudaError_t e = swept::raise_smem_limit((const void*)swept2d::k_tile2d<T, L>, smem);
   for (int64_t m = from; m < to && e == cudaSuccess; ++m) {
     const int kk = (int)(n * (m + 1) / total - n * m / total);
@@ -346,7 +347,7 @@ swept_status swept2d_init(const swept2d_config* cfg, swept2d_handle** out) {
     }
   }
   cudaGetLastError();  // clear a no-device error
-  if (cfg->tile_w == 0 && cfg->threads == 0 && !h->persistent)
+  if (cfg->tile_w == 0 && cfg->threads == 0 && !h->persistent && g.ntx * g.nty * g.Es >= g.nx * g.ny)
     h->tile = choose_overlap(cfg->nx, cfg->ny, cfg->dtype, h->sm_count > 0 ? h->sm_count : 152);
   *out = h;
   return SWEPT_OK;
