@@ -73,7 +73,7 @@ struct BatchDev {
 template <typename T, class Op>
 struct BatchCtx {
   static constexpr int kR = Op::R, kC = Op::C;
-  static constexpr bool kFixedTiers = sizeof(T) == 4;
+  static constexpr bool kPhaseTiers = has_phase<T, Op>();
   T* sm;
   Geom g;
   typename Op::K k;
@@ -99,11 +99,19 @@ struct BatchCtx {
   __device__ __forceinline__ void store_edge(int r, int c, int j, int64_t e) {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e, edge_slots(g) * g.E, dbg::EDGE)) e_out[e] = row(r, c)[j];
   }
-  // the per-problem kernels' tier code (strided, or paired for radius 2)
-  // FP32: all tiers of a phase with a fixed mapping of points to threads
-  __device__ __forceinline__ bool phase_tiers(int n, int lo0, int hi0, int d, int wall) {
-    return wall == NO_WALL && fixed_tiers<Op, 4>(sm, g.M, n, lo0, hi0, d, k);
+  __device__ __forceinline__ void begin_pass() {
+    if (sizeof(T) == 8) ks_begin(sm, g);
   }
+  // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
+  __device__ __forceinline__ bool phase_tiers(int n, int base, int lo0, int hi0, int d, int64_t , int wall) {
+    if constexpr (sizeof(T) == 8) {
+      if (phase_in_window<Op>(g.M, n, lo0, hi0, d)) ks_f64_phase(sm, g.M, n, base, lo0, hi0, d, k, gridDim.x, [](int, int, int) {});
+      return true;
+    } else {
+      return wall == NO_WALL && fixed_tiers<Op, 4>(sm, g.M, n, lo0, hi0, d, k);
+    }
+  }
+  // the per-problem kernels' tier code (strided, or paired for radius 2)
   __device__ __forceinline__ void level(int s, int, int lo, int hi, int64_t, int wall) {
     if (dbg::level(g.M, lo, hi, kR)) LevelImpl<T, Op>::run(sm, g.M, stage_c<Op>(s), s & 1, lo, hi, wall, 1, k);
     __syncthreads();

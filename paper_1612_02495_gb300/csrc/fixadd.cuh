@@ -26,6 +26,7 @@
 // Range: finite operands, exponents within 24 of each other, none zero or
 // subnormal, results that are not subnormal and not below 2^53 LSBs.
 #pragma once
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -315,6 +316,18 @@ SWFIX float float_bits(double x) {
   memcpy(&f, &b, 4);
   return f;
 #endif
+}
+
+// Whether second_fourth is likely to hold: operands in its range and differences above 2^-20 of the largest, in
+// single precision with the operands' bits cut off.  A guess, either way.
+SWFIX bool differ(double a, double b, double c, double d, double e) {
+  const uint32_t wa = mag(a), wb = mag(b), wc = mag(c), wd = mag(d), we = mag(e);
+  const uint32_t top = umax(umax(umax(wa, wb), umax(wd, we)), wc);
+  int E;
+  const bool in = in_range(umin(umin(umin(wa, wb), umin(wd, we)), wc), top, E);
+  const float fc = float_bits(c), s1 = float_bits(b) + float_bits(d), s2 = float_bits(a) + float_bits(e);
+  const float d2 = s1 - 2.f * fc, d4 = s2 - 4.f * s1 + 6.f * fc, least = float_bits(make_double(top, 0)) * 0x1p-20f;
+  return in && fabsf(d2) > least && fabsf(d4) > least;
 }
 
 }  // namespace fix

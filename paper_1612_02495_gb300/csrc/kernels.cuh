@@ -300,34 +300,98 @@ struct LevelImpl {
       scalar_level_any<T, Op, 1>(sm, M, out_row, lo, hi, wall, chunk, k);
   }
 };
+// contexts of these schemes run whole phases (phase_tiers): the scalar ones in FP32, KS in FP64
+template <typename T, class Op>
+constexpr bool has_phase() {
+  return Op::C == 1 && (sizeof(T) == 4 || Op::R == 2);
+}
+// debug build: the phase's widest tier is inside the window
+template <class Op>
+__device__ __forceinline__ bool phase_in_window(int M, int n, int lo0, int hi0, int d) {
+  const int s = d > 0 ? 1 : n;
+  return dbg::level(M, lo0 + d * s, max(hi0 - d * s, lo0 + d * s), Op::R);
+}
+
+// ---------------------------------------------------------------------------
 // KS in FP64: a tier's points on the integer and FP64 pipes together
 // (KsOp::point_int).  KS grids are periodic, so a window never holds a wall,
 // and chunk 2 has nothing to gain: one point already keeps both pipes busy.  A
 // point the integer arithmetic does not handle is left out in the first loop
-// and redone in FP64 after it (under 1 % of the warps on the KS workload), so
+// and computed in FP64 after it, so
 // that the loop has no branch and a warp's FP64 instructions start before its
 // integer chain has ended: with the branch at each point a lone warp took 1190
 // cycles a point, without 929.
-// Bound: FP64 and integer issue (58 % and 65 % of their pipes).  2^20 points,
+// Bound: FP64 and integer issue.  2^20 points,
 // tile 1024, 256 threads, persistent, 1,000 steps: 44.6 -> 26.0 ms.  Two points
 // a thread, sharing their operands' conversions, gave 25.3 ms there but took
 // 2^14 points (tile 128) from 3.85 to 4.22 ms (start: 4.06 ms); four spilled (36.6 ms); four or
 // five blocks a SM instead of three 27.2 and 28.3 ms.
+//
+// How many points fail is up to the field: on the noisy KS field 1 to 3 of a thousand
+// warp trips, at other points in every tier; on zeros, constants, one long wave or a small
+// wave on a large mean all of them in tier after tier, and then the attempt is lost work.  So the block's
+// failing warps keep a count (KsNote), and it goes over to FP64 for the rest of its pass when
+// that is the faster choice:
+//   - A launch that fills the GPU is bound by the FP64 and integer pipes: integers and a second run at some
+//     points cost more than FP64 alone when half of a tier's trips fail.
+//   - With at most two working warps a sub-partition a tier lasts as long as its slowest warp, 970 cycles a
+//     trip or, with a failing point, 2,030, where FP64 alone takes 1,040: one lost trip in eight is too many.
+// All of this runs where a point has failed; the others read one word every second tier.  Milliseconds (last:
+// FP64 alone), noisy field and constant one, before and with the count:
+//   2^20, tile 1024, 256 threads, persistent, 400 steps   10.35 / 26.5    10.4 / 18.2    18.3
+//   2^14, tile 128, 256 threads, 1,000 steps               1.94 / 4.19    1.99 / 2.05    2.06
+// A verdict by a vote or a counting barrier in every tier, every second one or after 2, 4, 8, ... took the
+// latter's noisy run to 2.08, 2.03 and 2.10: a pass launched by itself fetches its code anew, so that even
+// what runs once a phase costs a microsecond.
+// ---------------------------------------------------------------------------
+// Kept in positions 0 and 1 of window row 0, which no pass of a radius-2 scheme touches (a row starts with
+// R halo points, and only odd tiers insert an edge that far out).  Written in the odd tiers of a
+// pass, read in the even ones.
+struct KsNote {
+  unsigned lost;    // warp trips with a failing point in the odd tiers so far
+  unsigned fp64;    // not 0: FP64 from here on
+  unsigned now[2];  // those of this odd tier, by turns; each starts from 0, or from what a tier four
+                    // before it left when none failed in between
+};
+constexpr int kKsLoneWarps = 2 * 4 * 152;
+
+// at the start of a pass; FP64 where a thread makes more trips than ks_f64_tier has bits for
+__device__ __forceinline__ void ks_begin(void* row0, const Geom& g) {
+  if (threadIdx.x == 0) *reinterpret_cast<KsNote*>(row0) = KsNote{0, g.W + g.X > 32 * (int)blockDim.x, {}};
+}
+// one warp's `lost` trips in odd tier s of the pass, on a range of `points`
+__device__ __forceinline__ void ks_note(KsNote* note, unsigned lost, int s, int points, int64_t blocks) {
+  const int T = (int)blockDim.x, slot = (s >> 1) & 1;
+  note->now[slot ^ 1] = 0;
+  const unsigned now = atomicAdd(&note->now[slot], lost) + lost, all = atomicAdd(&note->lost, lost) + lost;
+  const bool lone = (int)min(blocks, (int64_t)kKsLoneWarps + 1) * ((min(T, points) + 31) >> 5) <= kKsLoneWarps;
+  // a single trip may fail on any field, but for the few points of a pass's first tier; a warp makes points / T
+  // trips a tier, at least one, in (s + 1) / 2 odd tiers
+  const unsigned least = s > 1 ? 2 : 1;
+  if (lone ? all >= least && 8 * all * T >= (unsigned)((s + 1) / 2 * max(points, T))
+           : now >= least && 64 * now >= (unsigned)points)
+    note->fp64 = 1;
+}
+// The points that the integer form did not handle: bit 0 of `failed` is the thread's last trip.  Called by the lanes
+// with one.
 template <int STAGE>
-__device__ __noinline__ void ks_f64_redo(const double* in, double* out, int lo, int hi, KsOp<double>::K k) {
-  for (int j = lo + (int)threadIdx.x; j < hi; j += (int)blockDim.x) {
-    const double p2 = STAGE == 1 ? out[j] : 0.0;
-    double r;
-    if (!KsOp<double>::point_int<STAGE>(in + j - 2, p2, k, r)) out[j] = KsOp<double>::point_fp<STAGE>(in + j - 2, p2, k);
+__device__ __noinline__ void ks_f64_redo(const double* in, double* out, int j, int hi, unsigned failed,
+                                         KsOp<double>::K k, KsNote* note, int s, int points, int64_t blocks) {
+  const int T = (int)blockDim.x;
+  if (STAGE == 0) {
+    const unsigned lanes = __activemask(), lost = __popc(__reduce_or_sync(lanes, failed));
+    if ((lanes & ((1u << (threadIdx.x & 31u)) - 1u)) == 0) ks_note(note, lost, s, points, blocks);
   }
+  while (j + T < hi) j += T;
+  for (; failed; failed >>= 1, j -= T)
+    if (failed & 1u) out[j] = KsOp<double>::point_fp<STAGE>(in + j - 2, STAGE == 1 ? out[j] : 0.0, k);
 }
 template <int STAGE>
-__device__ __forceinline__ void ks_f64_level(double* sm, int M, int out_row, int lo, int hi,
-                                             const KsOp<double>::K& k) {
-  const double* in = sm + (out_row ^ 1) * M;
-  double* out = sm + out_row * M;
-  bool bad = false;
-  for (int j = lo + (int)threadIdx.x; j < hi; j += (int)blockDim.x) {
+__device__ __forceinline__ void ks_f64_tier(const double* in, double* out, int lo, int hi, const KsOp<double>::K& k,
+                                            KsNote* note, int s, int64_t blocks) {
+  unsigned failed = 0;
+  const int first = lo + (int)threadIdx.x;
+  for (int j = first; j < hi; j += (int)blockDim.x) {
     double v[5];
 #pragma unroll
     for (int d = 0; d < 5; ++d) v[d] = in[j + d - 2];
@@ -335,20 +399,62 @@ __device__ __forceinline__ void ks_f64_level(double* sm, int M, int out_row, int
     double r;
     const bool ok = KsOp<double>::point_int<STAGE>(v, p2, k, r);
     if (ok) out[j] = r;
-    bad = bad || !ok;
+    failed = 2 * failed + (ok ? 0u : 1u);
   }
-  if (bad) ks_f64_redo<STAGE>(in, out, lo, hi, k);
+  if (failed) ks_f64_redo<STAGE>(in, out, first, hi, failed, k, note, s, hi - lo, blocks);
 }
-template <>
-struct LevelImpl<double, KsOp<double>> {
-  __device__ __forceinline__ static void run(double* sm, int M, int stage, int out_row, int lo, int hi, int /*wall*/,
-                                             int /*chunk*/, const KsOp<double>::K& k) {
-    if (stage == 0)
-      ks_f64_level<0>(sm, M, out_row, lo, hi, k);
-    else
-      ks_f64_level<1>(sm, M, out_row, lo, hi, k);
+template <int STAGE>
+__device__ __forceinline__ void ks_f64_tier_fp(const double* in, double* out, int lo, int hi,
+                                               const KsOp<double>::K& k) {
+  for (int j = lo + (int)threadIdx.x; j < hi; j += (int)blockDim.x)
+    out[j] = KsOp<double>::point_fp<STAGE>(in + j - 2, STAGE == 1 ? out[j] : 0.0, k);
+}
+// Tiers 1..n of a phase (base + 1.. of the pass), tier s on [lo + d s, hi - d s); after(s, lo, hi) when tier s is
+// complete.  `blocks`: of the launch that have a tile.
+template <class After>
+__device__ __forceinline__ void ks_f64_phase(double* sm, int M, int n, int base, int lo, int hi, int d,
+                                             const KsOp<double>::K& k, int64_t blocks, After&& after) {
+  double* row0 = sm;
+  double* row1 = sm + M;
+  KsNote* note = reinterpret_cast<KsNote*>(sm);
+  unsigned fp64 = d > 0 ? *(volatile unsigned*)&note->fp64 : 0;  // a growing phase starts with few points
+  int s = 1;
+  if (!fp64) {
+    for (; s + 1 <= n && !fp64; s += 2) {
+      lo += d, hi -= d;
+      ks_f64_tier<0>(row0, row1, lo, hi, k, note, base + s, blocks);
+      __syncthreads();
+      after(s, lo, hi);
+      fp64 = *(volatile unsigned*)&note->fp64;
+      lo += d, hi -= d;
+      ks_f64_tier<1>(row1, row0, lo, hi, k, note, base + s, blocks);
+      __syncthreads();
+      after(s + 1, lo, hi);
+    }
+    if (s <= n && !fp64) {
+      lo += d, hi -= d;
+      ks_f64_tier<0>(row0, row1, lo, hi, k, note, base + s, blocks);
+      __syncthreads();
+      after(s++, lo, hi);
+    }
   }
-};
+  for (; s + 1 <= n; s += 2) {  // s is odd: a pass changes over after an even tier
+    lo += d, hi -= d;
+    ks_f64_tier_fp<0>(row0, row1, lo, hi, k);
+    __syncthreads();
+    after(s, lo, hi);
+    lo += d, hi -= d;
+    ks_f64_tier_fp<1>(row1, row0, lo, hi, k);
+    __syncthreads();
+    after(s + 1, lo, hi);
+  }
+  if (s <= n) {
+    lo += d, hi -= d;
+    ks_f64_tier_fp<0>(row0, row1, lo, hi, k);
+    __syncthreads();
+    after(s, lo, hi);
+  }
+}
 // Euler: chunk 2 = two threads per face in the flux phase
 template <typename T>
 struct LevelImpl<T, EulerOp<T>> {
@@ -443,8 +549,7 @@ struct FixedTiers {
 template <class Op, int MAXQ>
 __device__ __forceinline__ bool fixed_tiers(float* sm, int M, int n, int lo0, int hi0, int d,
                                             const typename Op::K& k) {
-  const int sw = d > 0 ? 1 : n;  // the widest tier
-  if (!dbg::level(M, lo0 + d * sw, max(hi0 - d * sw, lo0 + d * sw), Op::R)) return true;
+  if (!phase_in_window<Op>(M, n, lo0, hi0, d)) return true;
   const int T = (int)blockDim.x, pairs = (M - 2 * (Op::R & ~1) + 1) / 2, need = (pairs + T - 1) / T;
   if ((M & 1) || need > MAXQ) return false;
   if (Op::R == 1 || ((lo0 | hi0) & 1)) {
@@ -494,7 +599,7 @@ struct DevCtx {
   using value_type = T;
   using op_type = Op;
   static constexpr int kR = Op::R, kC = Op::C;
-  static constexpr bool kFixedTiers = !TAPE && sizeof(T) == 4 && Op::C == 1;
+  static constexpr bool kPhaseTiers = has_phase<T, Op>() && !(TAPE && sizeof(T) == 4);
   T* sm;
   Geom g;
   typename Op::K k;
@@ -522,16 +627,29 @@ struct DevCtx {
   __device__ __forceinline__ void store_edge(int r, int c, int j, int64_t e) {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e, edge_slots(g) * g.E, dbg::EDGE)) e_out[e] = row(r, c)[j];
   }
-  // FP32: all tiers of a phase with a fixed mapping of points to threads
-  __device__ __forceinline__ bool phase_tiers(int n, int lo0, int hi0, int d, int wall) {
-    return wall == NO_WALL && fixed_tiers<Op, 4>(sm, g.M, n, lo0, hi0, d, k);
+  __device__ __forceinline__ void begin_pass() {
+    if (sizeof(T) == 8) ks_begin(sm, g);
+  }
+  // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
+  __device__ __forceinline__ bool phase_tiers(int n, int base, int lo0, int hi0, int d, int64_t origin, int wall) {
+    if constexpr (sizeof(T) == 8) {
+      if (phase_in_window<Op>(g.M, n, lo0, hi0, d)) ks_f64_phase(sm, g.M, n, base, lo0, hi0, d, k, gridDim.x, [&](int s, int lo, int hi) { record(s, base, lo, hi, origin); });
+      return true;
+    } else {
+      return wall == NO_WALL && fixed_tiers<Op, 4>(sm, g.M, n, lo0, hi0, d, k);
+    }
   }
   __device__ __forceinline__ void level(int s, int base, int lo, int hi, int64_t origin, int wall) {
     if (dbg::level(g.M, lo, hi, kR)) LevelImpl<T, Op>::run(sm, g.M, stage_c<Op>(s), s & 1, lo, hi, wall, g.chunk, k);
+    // the tier's mapping of points to threads (strided or paired)
+    // need not match the record's, so the tier must be complete first
+    if (TAPE) __syncthreads();
+    record(s, base, lo, hi, origin);
+    if (!TAPE) __syncthreads();
+  }
+  // a complete tier's values onto the tape
+  __device__ __forceinline__ void record(int s, int base, int lo, int hi, int64_t origin) {
     if (TAPE) {
-      // the tier's mapping of points to threads (strided or paired)
-      // need not match this loop's, so the tier must be complete first
-      __syncthreads();
       const int64_t slot = tape.base + base + s - tape.tier0;
       if (slot >= 0 && slot < tape.ntiers)
         for (int j = lo + (int)threadIdx.x; j < hi; j += (int)blockDim.x) {
@@ -539,8 +657,8 @@ struct DevCtx {
 #pragma unroll
           for (int c = 0; c < Op::C; ++c) tape.p[(slot * Op::C + c) * g.N + x] = row(s & 1, c)[j];
         }
+      __syncthreads();
     }
-    __syncthreads();
   }
 };
 
@@ -565,7 +683,7 @@ struct RegCtx : Base {
   using Op = typename Base::op_type;
   static constexpr int R = Op::R;
   static_assert(Op::C == 1 && P >= 1, "register tiers need a scalar scheme");
-  static constexpr bool kFixedTiers = false;  // its own level() keeps the whole pass in registers
+  static constexpr bool kPhaseTiers = false;  // its own level() keeps the whole pass in registers
   T a[P], b[P];            // rows 0 (even tiers) and 1 (odd tiers)
   T ha[2 * R], hb[2 * R];  // halo of rows 0 / 1: [0, R) -> points 0..R-1, [R, 2R) -> points W+R..W+2R-1
   bool in_regs;
@@ -729,7 +847,7 @@ struct PDevCtx {
   using value_type = T;
   using op_type = Op;
   static constexpr int kR = Op::R, kC = Op::C;
-  static constexpr bool kFixedTiers = sizeof(T) == 4 && Op::C == 1;
+  static constexpr bool kPhaseTiers = has_phase<T, Op>();
   T* sm;
   Geom g;
   typename Op::K k;
@@ -755,9 +873,17 @@ struct PDevCtx {
   __device__ __forceinline__ void store_edge(int r, int c, int j, int64_t e) {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e, edge_slots(g) * g.E, dbg::EDGE)) e_out[e] = row(r, c)[j];
   }
-  // FP32: all tiers of a phase with a fixed mapping of points to threads
-  __device__ __forceinline__ bool phase_tiers(int n, int lo0, int hi0, int d, int wall) {
-    return wall == NO_WALL && fixed_tiers_call<Op>(g.M, n, lo0, hi0, d, k);
+  __device__ __forceinline__ void begin_pass() {
+    if (sizeof(T) == 8) ks_begin(sm, g);
+  }
+  // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
+  __device__ __forceinline__ bool phase_tiers(int n, int base, int lo0, int hi0, int d, int64_t , int wall) {
+    if constexpr (sizeof(T) == 8) {
+      if (phase_in_window<Op>(g.M, n, lo0, hi0, d)) ks_f64_phase(sm, g.M, n, base, lo0, hi0, d, k, min((int64_t)gridDim.x, g.nt), [](int, int, int) {});
+      return true;
+    } else {
+      return wall == NO_WALL && fixed_tiers_call<Op>(g.M, n, lo0, hi0, d, k);
+    }
   }
   __device__ __forceinline__ void level(int s, int, int lo, int hi, int64_t, int wall) {
     if (dbg::level(g.M, lo, hi, kR)) LevelImpl<T, Op>::run(sm, g.M, stage_c<Op>(s), s & 1, lo, hi, wall, g.chunk, k);
@@ -843,7 +969,7 @@ struct ClusterCtx {
   using value_type = T;
   using op_type = Op;
   static constexpr int kR = Op::R, kC = Op::C;
-  static constexpr bool kFixedTiers = sizeof(T) == 4 && Op::C == 1;
+  static constexpr bool kPhaseTiers = has_phase<T, Op>();
   T* sm;         // the block's window rows (and Euler scratch)
   T* ex_in;      // export area of the previous pass (read remotely)
   T* ex_out;     // export area this pass writes (own tile's edges)
@@ -874,9 +1000,17 @@ struct ClusterCtx {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e - (int64_t)my_rank * g.E, g.E, dbg::EDGE))
       ex_out[e - (int64_t)my_rank * g.E] = row(r, c)[j];
   }
-  // FP32: all tiers of a phase with a fixed mapping of points to threads
-  __device__ __forceinline__ bool phase_tiers(int n, int lo0, int hi0, int d, int wall) {
-    return wall == NO_WALL && fixed_tiers_call<Op>(g.M, n, lo0, hi0, d, k);
+  __device__ __forceinline__ void begin_pass() {
+    if (sizeof(T) == 8) ks_begin(sm, g);
+  }
+  // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
+  __device__ __forceinline__ bool phase_tiers(int n, int base, int lo0, int hi0, int d, int64_t , int wall) {
+    if constexpr (sizeof(T) == 8) {
+      if (phase_in_window<Op>(g.M, n, lo0, hi0, d)) ks_f64_phase(sm, g.M, n, base, lo0, hi0, d, k, gridDim.x, [](int, int, int) {});
+      return true;
+    } else {
+      return wall == NO_WALL && fixed_tiers_call<Op>(g.M, n, lo0, hi0, d, k);
+    }
   }
   __device__ __forceinline__ void level(int s, int, int lo, int hi, int64_t, int wall) {
     if (dbg::level(g.M, lo, hi, kR)) LevelImpl<T, Op>::run(sm, g.M, stage_c<Op>(s), s & 1, lo, hi, wall, g.chunk, k);

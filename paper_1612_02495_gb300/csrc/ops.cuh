@@ -96,18 +96,29 @@ struct KsOp {
     r = fma_rn(STAGE == 0 ? k.mdth : k.mdt, combine(v[3], um2, d2, d4, k), STAGE == 0 ? v[2] : prev2);
     return lin && sq;
   }
-  // the FP64 instructions out of line: a call is never turned into predicated instructions
-  template <int STAGE>
-  __device__ __noinline__ static T point_cold(T a, T b, T c, T d, T e, T prev2, K k) {
-    const T v[5] = {a, b, c, d, e};
-    return point_fp<STAGE>(v, prev2, k);
+  // u_{i-1}^2 and the two differences in FP64, out of line: a call is never turned into
+  // predicated instructions
+  struct Parts {
+    T um2, d2, d4;
+  };
+  __device__ __noinline__ static Parts parts_fp(T a, T b, T c, T d, T e) {
+    const T sp1 = add_rn(d, b), sp2 = add_rn(e, a);
+    return Parts{mul_rn(b, b), fma_rn(T(-2), c, sp1), fma_rn(T(6), c, fma_rn(T(-4), sp1, sp2))};
   }
+  // One point by itself (the classic kernels, whose warps keep nothing from one sub-timestep to the
+  // next).  The integer form is tried where it is likely to hold for the whole warp: operands in its
+  // range, and differences that do not vanish beside them in single precision (bits cut off, no FP64
+  // instruction).  The branch for a point that fails all the same comes before the common end, so that it
+  // issues the eleven FP64 operations once.
   template <int STAGE>
   __device__ __forceinline__ static T point(const T* v, T prev2, const K& k) {
     if constexpr (sizeof(T) == 8) {
-      T r;
-      if (!point_int<STAGE>(v, prev2, k, r)) r = point_cold<STAGE>(v[0], v[1], v[2], v[3], v[4], prev2, k);
-      return r;
+      if (!__all_sync(__activemask(), fix::differ(v[0], v[1], v[2], v[3], v[4]))) return point_fp<STAGE>(v, prev2, k);
+      Parts p;
+      const bool lin = fix::second_fourth(v[0], v[1], v[2], v[3], v[4], p.d2, p.d4);
+      const bool sq = fix::square(v[1], p.um2);
+      if (!(lin && sq)) p = parts_fp(v[0], v[1], v[2], v[3], v[4]);
+      return fma_rn(STAGE == 0 ? k.mdth : k.mdt, combine(v[3], p.um2, p.d2, p.d4, k), STAGE == 0 ? v[2] : prev2);
     } else {
       return point_fp<STAGE>(v, prev2, k);
     }

@@ -15,7 +15,7 @@
 //                                  compute sub-timestep (base + s) on [lo, hi)
 //                                  into row s&1 from row (s-1)&1 (and row s&1
 //                                  for the second stage), then sync
-//   kFixedTiers (optional)           the context has phase_tiers (run_phase)
+//   kPhaseTiers (optional)           the context has phase_tiers (run_phase)
 //   kSlab (optional, with member `sl`)
 //                                  the context runs one slab of a grid split
 //                                  over ranks: edge indices go to the slab's
@@ -62,19 +62,24 @@ SW_HD void for_tiers(int n, F&& f) {
   if (s <= n) f(s);
 }
 
-// Contexts with kFixedTiers have phase_tiers(n, lo0, hi0, d, wall): all n tiers of a
-// phase at once, or false with nothing done.
+// Contexts with kPhaseTiers have begin_pass(), called before the window is filled, and
+// phase_tiers(n, base, lo0, hi0, d, origin, wall): all n tiers of a phase at once, or false with nothing done.
 template <class Cx, class = void>
 struct has_phase_tiers : std::false_type {};
 template <class Cx>
-struct has_phase_tiers<Cx, std::enable_if_t<Cx::kFixedTiers>> : std::true_type {};
+struct has_phase_tiers<Cx, std::enable_if_t<Cx::kPhaseTiers>> : std::true_type {};
 
-// all tiers s = 1..n of a phase on [lo0 + d s, hi0 - d s) (d = R shrinks, -R
-// grows) where the context can; false: they are still to be run, one by one
 template <class Cx>
-SW_HD bool run_phase(Cx& cx, int n, int lo0, int hi0, int d, int wall) {
+SW_HD void begin_pass(Cx& cx) {
+  if constexpr (has_phase_tiers<Cx>::value) cx.begin_pass();
+}
+
+// all tiers s = 1..n of a phase (sub-timesteps base + s) on [lo0 + d s, hi0 - d s) (d = R
+// shrinks, -R grows) where the context can; false: they are still to be run, one by one
+template <class Cx>
+SW_HD bool run_phase(Cx& cx, int n, int base, int lo0, int hi0, int d, int64_t origin, int wall) {
   if constexpr (has_phase_tiers<Cx>::value)
-    return cx.phase_tiers(n, lo0, hi0, d, wall);
+    return cx.phase_tiers(n, base, lo0, hi0, d, origin, wall);
   else
     return false;
 }
@@ -91,12 +96,13 @@ SW_HD void run_up(Cx& cx, const Geom& g_in, int64_t b, int hh, bool write_top) {
   const int w = tile_width(g, b);
   const int64_t x0 = b * (int64_t)g.W;
   const int64_t origin = x0 - g.R;
+  begin_pass(cx);
   cx.for_range(0, w * g.C, [&](int i) {
     const int c = g.C == 1 ? 0 : i / w, k = i - c * w;
     cx.load_u(0, c, g.R + k, x0 + k);
   });
   cx.sync();
-  if (!run_phase(cx, hh, g.R, g.R + w, g.R, NO_WALL))
+  if (!run_phase(cx, hh, 0, g.R, g.R + w, g.R, origin, NO_WALL))
     for_tiers(hh, [&](int s) { cx.level(s, 0, g.R + g.R * s, g.R + w - g.R * s, origin, NO_WALL); });
   const int per_level = g.C * 2 * g.R;
   const int per_side = hh * per_level;
@@ -150,6 +156,7 @@ SW_HD void run_diamond(Cx& cx, const Geom& g_in, int64_t b, int odd, int mode, i
   const int64_t tr = right_tile(g, odd, b);
   const int per_level = g.C * 2 * g.R;
   const int per_side = hh * per_level;
+  begin_pass(cx);
   cx.for_range(0, 2 * per_side, [&](int i) {
     const int which = i >= per_side ? 1 : 0;  // 0: right edges of the left tile, 1: left edges of the right tile
     const int rem = i - which * per_side;
@@ -169,11 +176,11 @@ SW_HD void run_diamond(Cx& cx, const Geom& g_in, int64_t b, int odd, int mode, i
   }
   cx.sync();
   const int wall = window_wall(g, origin, w + 2 * g.R);
-  if (!run_phase(cx, hh, dofs + grow_lo(g, 0), dofs + grow_hi(g, 0), -g.R, wall))
+  if (!run_phase(cx, hh, 0, dofs + grow_lo(g, 0), dofs + grow_hi(g, 0), -g.R, origin, wall))
     for_tiers(hh, [&](int s) { cx.level(s, 0, dofs + grow_lo(g, s), dofs + grow_hi(g, s), origin, wall); });
   if (mode == MODE_DIAMOND) {
     const int top = wide ? g.h : g.h - 1;  // a triangle's tier h is empty; a wide tile's is its flat top
-    if (!run_phase(cx, top, g.R, g.R + w, g.R, wall))
+    if (!run_phase(cx, top, g.h, g.R, g.R + w, g.R, origin, wall))
       for_tiers(top, [&](int s) { cx.level(s, g.h, g.R + g.R * s, g.R + w - g.R * s, origin, wall); });
     const int per_side_h = g.h * per_level;
     cx.for_range(0, 2 * per_side_h, [&](int i) {
