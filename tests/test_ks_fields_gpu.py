@@ -132,3 +132,47 @@ def test_cost(S, n, steps, most, run, plan):
             ms.setdefault(kind, []).append(a.elapsed_time(b))
         sol.close()
     assert min(ms["constant"][1:]) < most * min(ms["noisy"][1:]), ms
+
+
+# ---- adjoint: the same with the cotangent, dL/dnu within the bound of test_adjoint_gpu.py ----
+def adjoint_run(S, u0, gT, steps, **kw):
+    import torch
+
+    sol = S.Solver(S.KS, S.F64, u0.size, DX, DT, NU, **kw)
+    ckpt = torch.empty(sol.ckpt_size(steps), dtype=torch.uint8, device="cuda")
+    u, g = torch.from_numpy(u0).cuda(), torch.from_numpy(gT).cuda()
+    sol.forward_ckpt(u, steps, ckpt)
+    ms = []
+    for _ in range(4):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        gu, gp = sol.adjoint(g, steps, ckpt)
+        b.record()
+        torch.cuda.synchronize()
+        ms.append(a.elapsed_time(b))
+    sol.sync_status()
+    sol.close()
+    return u.cpu().numpy(), gu.cpu().numpy(), float(gp.cpu().numpy()[0]), min(ms[1:])
+
+
+@pytest.mark.parametrize("ukind,gkind", [("constant", "onehot"), ("mixed", "onehot"), ("packet", "packet"), ("zero", "short"),
+                                         ("mixed", "zero"), ("short", "constant"), ("wide", "wide"), ("mixed", "mixed")])
+@pytest.mark.parametrize("n,kw", [(512, dict(tile_w=64)), (1027, dict(tile_w=128, threads=32)), (1009, dict()),
+                                  (2 * 2048 + 8, dict(tile_w=2048, threads=32))])
+def test_adjoint(S, n, kw, ukind, gkind):
+    steps = 37
+    u0, gT = field(ukind, n), field(gkind, n)
+    u, g, gnu, _ = adjoint_run(S, u0, gT, steps, **kw)
+    rg, rnu, cond = oracle.ks_adjoint(u0, DX, DT, NU, steps, gT, with_condition=True, threads=8)
+    assert same(u, oracle.ks(u0, DX, DT, NU, steps, threads=8))
+    assert np.array_equal(g, rg)
+    assert abs(gnu - rnu) <= 1e-12 * abs(rnu) + 8 * 2.0 ** -52 * cond
+
+
+# 17 or 18 FP64 operations a point instead of 11 or 12; running both forms took 2.2 times as long
+def test_adjoint_cost(S):
+    n, steps = 1 << 18, 50
+    u0, g = field("constant", n), np.random.Generator(np.random.Philox(5)).standard_normal(n)
+    noisy = adjoint_run(S, inputs.ks_problem(n=n)["u0"], g, steps, tile_w=512, threads=256)[3]
+    ones = adjoint_run(S, u0, np.ones(n), steps, tile_w=512, threads=256)[3]
+    assert ones < 1.7 * noisy, (ones, noisy)
