@@ -83,7 +83,7 @@ int choose_tile(int64_t nx, int64_t ny, int dtype) {
 // L in {2, 4, 8} and G in {1..8} on 256^2 to 4096^2 points, within 10 % of
 // the larger ones.  Microseconds a step, the best shape against the swept default (tile 32):
 //   FP32  256^2 0.66 / 2.14   1024^2 1.50 / 6.99   4096^2 18.9 / 105
-//   FP64  256^2 2.30 / 3.51   768 x 512 5.68 / 8.43   1024^2 12.9 / 14.5   4096^2 167 / 198
+//   FP64  256^2 2.08 / 3.49   768 x 512 4.91 / 7.08   1024^2 11.4 / 14.4   4096^2 165 / 198
 swept2d::Tile2d choose_overlap(int64_t nx, int64_t ny, int dtype, int sms) {
   swept2d::Tile2d best;
   double best_t = 1e300;

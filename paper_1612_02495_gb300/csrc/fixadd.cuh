@@ -188,17 +188,36 @@ SWFIX F96 round53(F96 x) {
   y.l &= ~low_ones(q + 1);
   return y;
 }
-// X rounded to 53 significant bits, as a double; ok is cleared when |X| < 2^53
-SWFIX double to_double(F96 x, int E, bool& ok) {
-  const uint32_t sg = (uint32_t)(x.h >> 31);
-  F96 y = sub(F96{x.l ^ sg, x.m ^ sg, (int32_t)((uint32_t)x.h ^ sg)}, F96{sg, sg, (int32_t)sg});
-  const int f = lead127(shr64(y.m, (uint32_t)y.h, 21));
-  ok = ok && f != 0;
+// |X| and its sign (all ones or 0)
+SWFIX F96 magnitude(F96 x, uint32_t& sg) {
+  sg = (uint32_t)(x.h >> 31);
+  return sub(F96{x.l ^ sg, x.m ^ sg, (int32_t)((uint32_t)x.h ^ sg)}, F96{sg, sg, (int32_t)sg});
+}
+// y = |X| >= 2^53 rounded to 53 significant bits; f from y's bits 53..84 (lead127)
+SWFIX double to_double_large(F96 y, uint32_t sg, int f, int E) {
   const int q = f - 127, r = q + 1;
   y = add_small(y, low_ones(q) + ((y.l >> (r & 31)) & 1u));
   const uint32_t lo = shr64(y.l, y.m, r & 31), hi = shr64(y.m, (uint32_t)y.h, r & 31);
   // the significand's bit 52 (or 53, after a carry) adds itself to the exponent field
   return make_double((hi + ((uint32_t)(E - kG + q) << 20)) | (sg & 0x80000000u), lo);
+}
+// X rounded to 53 significant bits, as a double; ok is cleared when |X| < 2^53
+SWFIX double to_double(F96 x, int E, bool& ok) {
+  uint32_t sg;
+  const F96 y = magnitude(x, sg);
+  const int f = lead127(shr64(y.m, (uint32_t)y.h, 21));
+  ok = ok && f != 0;
+  return to_double_large(y, sg, f, E);
+}
+// The same with X = 0 let through, as +0.
+SWFIX double to_double_or_zero(F96 x, int E, bool& ok) {
+  uint32_t sg;
+  const F96 y = magnitude(x, sg);
+  const int f = lead127(shr64(y.m, (uint32_t)y.h, 21));
+  const bool zero = (y.l | y.m | (uint32_t)y.h) == 0u;
+  ok = ok && (f != 0 || zero);
+  const double r = to_double_large(y, sg, f, E);
+  return zero ? 0.0 : r;
 }
 
 SWFIX uint32_t umin(uint32_t a, uint32_t b) { return a < b ? a : b; }
@@ -232,14 +251,12 @@ SWFIX bool second_fourth(double a, double b, double c, double d, double e, doubl
   return ok;
 }
 
-// Neighbour sums of a run of L points v of one column, with the points above and
+// ---- neighbour sums of a run of L points v of one column, with the points above and
 // below the run and the rows' neighbours w[i ST], e[i ST] (ST their stride):
-//   s[i] = (w_i + e_i) + (v_{i-1} + v_{i+1}), each sum correctly rounded.
-// One scale for the run, so a column value is converted once for the two sums it is
-// in.  False (s meaningless) when any value is outside the range.
+//   s[i] = (w_i + e_i) + (v_{i-1} + v_{i+1}), each sum correctly rounded ----
+// E for the run; false when a value is outside the range
 template <int L, int ST>
-SWFIX bool cross_sums(const double* w, const double* e, double up, double down, const double (&v)[L],
-                      double (&s)[L]) {
+SWFIX bool cross_scale(const double* w, const double* e, double up, double down, const double (&v)[L], int& E) {
   uint32_t lo = umin(mag(up), mag(down)), hi = umax(mag(up), mag(down));
 #pragma unroll
   for (int i = 0; i < L; ++i) {
@@ -247,18 +264,54 @@ SWFIX bool cross_sums(const double* w, const double* e, double up, double down, 
     lo = umin(lo, umin(a, umin(b, c)));
     hi = umax(hi, umax(a, umax(b, c)));
   }
-  int E;
-  bool ok = in_range(lo, hi, E);
+  return in_range(lo, hi, E);
+}
+// The same with zeros let through, as X = 0 at any scale; not -0, as an exact sum of 0 is taken for +0.
+template <int L, int ST>
+SWFIX bool cross_scale_zeros(const double* w, const double* e, double up, double down, const double (&v)[L], int& E) {
+  uint32_t lo = 0xffffffffu, hi = 0;
+  bool minus = false;
+  auto with = [&](double x) {
+    const uint32_t h = dhi(x);
+    const bool z = ((h << 1) | dlo(x)) == 0u;
+    lo = umin(lo, z ? 0xffffffffu : mag(x));
+    hi = umax(hi, mag(x));
+    minus = minus || (z && h != 0u);
+  };
+  with(up);
+  with(down);
+#pragma unroll
+  for (int i = 0; i < L; ++i) {
+    with(v[i]);
+    with(w[i * ST]);
+    with(e[i * ST]);
+  }
+  if (lo == 0xffffffffu) lo = hi = (uint32_t)kEmin << 20;  // nothing but zeros
+  return in_range(lo, hi, E) && !minus;
+}
+// The sums, on one scale for the run, so a column value is converted once for the two sums it is in; ok is
+// cleared when one is below 2^53 LSBs, but not 0.
+template <int L, int ST>
+SWFIX void cross_at(const double* w, const double* e, double up, double down, const double (&v)[L], double (&s)[L],
+                    int E, bool& ok) {
   const int sh0 = kG - E;
   F96 below = load(up, sh0), own = load(v[0], sh0);
 #pragma unroll
   for (int i = 0; i < L; ++i) {
     const F96 above = load(i + 1 < L ? v[i + 1] : down, sh0);
     const F96 sx = round53(add(load(w[i * ST], sh0), load(e[i * ST], sh0)));
-    s[i] = to_double(add(sx, round53(add(below, above))), E, ok);
+    s[i] = to_double_or_zero(add(sx, round53(add(below, above))), E, ok);
     below = own;
     own = above;
   }
+}
+// All of it: false (s meaningless) when a value or a sum is outside the range.
+template <int L, int ST>
+SWFIX bool cross_sums(const double* w, const double* e, double up, double down, const double (&v)[L],
+                      double (&s)[L]) {
+  int E;
+  bool ok = cross_scale<L, ST>(w, e, up, down, v, E) || cross_scale_zeros<L, ST>(w, e, up, down, v, E);
+  cross_at<L, ST>(w, e, up, down, v, s, E, ok);
   return ok;
 }
 

@@ -16,7 +16,9 @@
 // Bound: FP32, shared-memory instructions (3 a point at one a cycle and SM); FP64,
 // integer issue.  Measured against the swept passes with no plan set: 1024^2
 // FP32, 500 steps, 3.50 -> 0.75 ms; 768 x 512 FP64 insulated, 300 steps, 2.52 ->
-// 1.75 ms; with all five operations on the FP64 pipe 2.07 ms.
+// 1.44 ms; with all five operations on the FP64 pipe 2.07 ms.  Periodic FP64, 300 steps, noisy field / hot spot on
+// zeros / a field of subnormals (FP64 alone): 768 x 512 1.47 / 1.69 / 2.2 ms (swept passes 2.12), 1024^2 3.41 / 3.75 /
+// 5.0 (4.32).
 #pragma once
 #include "kernels2d.cuh"
 
@@ -50,28 +52,38 @@ __device__ __forceinline__ void tile2d_run_fp(const T* w, const T* e, T up, T do
   }
 }
 // In FP64 the three sums run on the integer pipes (fixadd.cuh), two of a point's
-// five operations on the FP64 pipe; a run with a value outside their range (a zero, a
-// magnitude 2^24 below another's) takes the FP64 instructions, behind a
-// branch the compiler cannot turn into predicated instructions: those would hold
-// the pipe as long as ones that run.
+// five operations on the FP64 pipe; a warp with a run outside their range (magnitudes more than 2^24
+// apart, a subnormal, -0, ...) takes the FP64 instructions, which cost it the same for one lane as for all.
+// The range is looked at before any sum, so such a warp pays for one form only, and the multiply-adds of a
+// point start while the sums of the next are formed; zeros, which a field may be full of, are looked at again and
+// stay with the integers.  What is left are sums that cancel to 2^-26 of their operands: those lanes do
+// their run again from the values in shared memory (`own`), behind a branch the compiler cannot turn into
+// predicated instructions: those would hold the pipe as long as ones that run.
 template <typename T, int L>
-__device__ __forceinline__ void tile2d_run(const T* w, const T* e, T up, T down, T (&v)[L], const Heat2dK<T>& k) {
+__device__ __forceinline__ void tile2d_run(const T* own, const T* w, const T* e, T up, T down, T (&v)[L],
+                                           const Heat2dK<T>& k) {
   if constexpr (sizeof(T) == 8) {
-    T s[L];
-    const bool ok = swept::fix::cross_sums<L, kTileWX>(w, e, up, down, v, s);
-    int redo = ok ? 0 : 1;
-    asm volatile("" : "+r"(redo));
-    if (redo == 0) {
+    int E;
+    bool in = swept::fix::cross_scale<L, kTileWX>(w, e, up, down, v, E);
+    if (!__all_sync(0xffffffffu, in)) in = swept::fix::cross_scale_zeros<L, kTileWX>(w, e, up, down, v, E);
+    if (__all_sync(0xffffffffu, in)) {
+      T s[L];
+      bool ok = true;
+      swept::fix::cross_at<L, kTileWX>(w, e, up, down, v, s, E, ok);
 #pragma unroll
       for (int i = 0; i < L; ++i) v[i] = fma_rn(k.fo, s[i], mul_rn(k.c1, v[i]));
+      int redo = ok ? 0 : 1;
+      asm volatile("" : "+r"(redo));
+      for (; redo > 0; --redo) {
+        asm volatile("" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < L; ++i) v[i] = own[i * kTileWX];
+        tile2d_run_fp<T, L>(w, e, up, down, v, k);
+      }
+      return;
     }
-    for (; redo > 0; --redo) {
-      asm volatile("" ::: "memory");
-      tile2d_run_fp<T, L>(w, e, up, down, v, k);
-    }
-  } else {
-    tile2d_run_fp<T, L>(w, e, up, down, v, k);
   }
+  tile2d_run_fp<T, L>(w, e, up, down, v, k);
 }
 
 template <typename T, int L>
@@ -101,7 +113,7 @@ __global__ void __launch_bounds__(kTileWX* kTileBands) k_tile2d(int64_t nx, int6
     const T* a = sm + (t & 1) * SIZE;
     T* b = sm + ((t & 1) ^ 1) * SIZE;
     const T up = r0 == 0 ? v[0] : a[at - ST], down = r0 + L == WY ? v[L - 1] : a[at + L * ST];
-    tile2d_run<T, L>(a + at + west, a + at + east, up, down, v, k);
+    tile2d_run<T, L>(a + at, a + at + west, a + at + east, up, down, v, k);
     if (t + 1 < kk) {
 #pragma unroll
       for (int i = 0; i < L; ++i) b[at + i * ST] = v[i];
