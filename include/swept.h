@@ -84,7 +84,9 @@ typedef enum {
  *            0 = chosen by the library (a divisor of n when one gives enough
  *            tiles).  Must be a multiple of 4*r (r = 1 heat, 2 KS/Euler), so
  *            that the half-cycle h = W/(2r) is even, with n >= 2 W.  The cluster
- *            and warp_tiles modes need W to divide n.
+ *            and warp_tiles modes need W to divide n.  The library's choice is
+ *            at least 128 to 256 points on small grids, but for these two modes
+ *            narrower where the wider tile is not legal in them.
  *   threads  threads per block, 0 = chosen by the library (<= 1024, multiple of 32)
  *   chunk    heat and KS: 1 = one point per thread per trip through a tier
  *            (strided; in FP32, radius-2 tiers take aligned pairs of points,

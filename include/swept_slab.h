@@ -39,7 +39,7 @@
  *
  * Limits: nranks <= nt; per-pass launches only (the config's persistent and
  * cluster must be 0); the plan (tile, threads, chunk, warp_tiles) is chosen as
- * by swept_init.  Every call returns a swept_status and never throws.
+ * by swept_init, but for tile_w = 0 no wider than leaves each rank a tile.  Every call returns a swept_status and never throws.
  */
 #ifndef SWEPT_SLAB_H
 #define SWEPT_SLAB_H

@@ -72,25 +72,48 @@ int narrowest_tile(int64_t n, int scheme, int dtype) {
 // still gives at least two blocks per SM; else at least one per SM; else the
 // smallest such W.  When no multiple of 4R divides n, the same rules choose
 // among all legal widths (the last tile then carries the n mod W extra points).
-// A width below `narrowest` (at most n / 2) gives way to the smallest
-// dividing width of up to twice that, or to that width itself.
-int choose_tile(int64_t n, int R, int sms, int narrowest) {
-  int W = 0;
-  for (int pass = 0; pass < 2 && !W; ++pass) {
+int choose_tile(int64_t n, int R, int sms) {
+  for (int pass = 0; pass < 2; ++pass) {
     auto ok = [&](int w) { return pass == 0 ? tile_divides(n, w, R) : tile_ok(n, w, R); };
+    int W = 0;
     for (int w = 4 * R; w <= 1024; w += 4 * R)
       if (ok(w) && n / w >= 2 * sms) W = w;
-    if (W) break;
+    if (W) return W;
     for (int w = 4 * R; w <= 1024; w += 4 * R)
       if (ok(w) && n / w >= sms) W = w;
     for (int w = 4 * R; w <= 4096 && !W; w += 4 * R)
       if (ok(w)) W = w;
+    if (W) return W;
   }
-  const int least = (int)std::min<int64_t>(narrowest, n / 2) / (4 * R) * (4 * R);
+  return 0;
+}
+// A width below `narrowest` (at most n / 2, and n / parts where a grid split over ranks needs a
+// tile for each) gives way to the smallest dividing width of up to twice that, or to that width itself.
+int widen_tile(int64_t n, int R, int W, int narrowest, int parts) {
+  const int most = (int)std::min<int64_t>(n / std::max(parts, 2), 1 << 30);
+  const int least = std::min(narrowest, most) / (4 * R) * (4 * R);
   if (W == 0 || W >= least) return W;
-  for (int w = least; w <= 2 * least; w += 4 * R)
+  for (int w = least; w <= std::min(2 * least, most); w += 4 * R)
     if (tile_divides(n, w, R)) return w;
   return least;
+}
+
+bool warp_tile(int64_t n, int W) {
+  const int P = W / 32;
+  return W % 32 == 0 && n % W == 0 && (P == 1 || P == 2 || P == 4 || P == 8);
+}
+constexpr int kMaxClusterTiles = 16;
+
+// The library's choice for a plan.  Warp tiles have four widths and a cluster few tiles, all alike: where the
+// wider tile is none of these the narrower one stays.
+int default_tile(const swept_config* cfg, int R, int sms, int parts) {
+  const int64_t n = cfg->n;
+  const int plain = choose_tile(n, R, sms);
+  const int wide = widen_tile(n, R, plain, narrowest_tile(n, cfg->scheme, cfg->dtype), parts);
+  if (wide == plain) return plain;
+  if (cfg->warp_tiles == 1 && !warp_tile(n, wide)) return plain;
+  if (cfg->cluster == 1 && (n % wide != 0 || n / wide > kMaxClusterTiles)) return plain;
+  return wide;
 }
 
 // The resident kernel (resident.cuh) for an n-point grid, or P = 0 where the
@@ -362,7 +385,13 @@ swept_status forward_ckpt(swept_handle* h, void* u, int64_t nsteps, char* ck, si
 
 extern "C" {
 
-swept_status swept_init(const swept_config* cfg, swept_handle** out) {
+swept_status swept_init(const swept_config* cfg, swept_handle** out) { return swept::make_plan(cfg, 1, out); }
+
+}  // extern "C"
+
+namespace swept {
+
+swept_status make_plan(const swept_config* cfg, int parts, swept_handle** out) {
   if (!cfg || !out) return SWEPT_EINVAL;
   *out = nullptr;
   const SchemeImpl* im = pick_impl(cfg->scheme, cfg->dtype);
@@ -394,7 +423,7 @@ swept_status swept_init(const swept_config* cfg, swept_handle** out) {
   cudaGetLastError();  // clear a no-device error
   cudaError_t e = cudaSuccess;
   const int R = im->R;
-  const int W = cfg->tile_w > 0 ? cfg->tile_w : choose_tile(cfg->n, R, h->sm_count, narrowest_tile(cfg->n, cfg->scheme, cfg->dtype));
+  const int W = cfg->tile_w > 0 ? cfg->tile_w : default_tile(cfg, R, h->sm_count, parts);
   // an explicit tile must be legal; with the library's choice, a grid too
   // small for two tiles of 4R points still gets a handle for classic_step_n
   if (cfg->tile_w != 0 && (cfg->tile_w < 0 || !tile_ok(cfg->n, W, R))) {
@@ -435,13 +464,11 @@ swept_status swept_init(const swept_config* cfg, swept_handle** out) {
     return SWEPT_EINVAL;
   }
   if (cfg->warp_tiles == 1) {
-    const int P = W / 32;
-    if (!h->tiled || g.X != 0 || im->C != 1 || W % 32 != 0 || (P != 1 && P != 2 && P != 4 && P != 8) ||
-        g.chunk != 1 || (cfg->threads != 0 && cfg->threads != 32)) {
+    if (!h->tiled || im->C != 1 || !warp_tile(cfg->n, W) || g.chunk != 1 || (cfg->threads != 0 && cfg->threads != 32)) {
       delete h;
       return SWEPT_EINVAL;
     }
-    g.P = P;
+    g.P = W / 32;
     th = 32;
   }
   h->threads = th;
@@ -473,7 +500,7 @@ swept_status swept_init(const swept_config* cfg, swept_handle** out) {
     delete h;
     return SWEPT_EINVAL;
   }
-  if (h->cluster && (g.nt > 16 || g.X != 0 || h->persistent ||
+  if (h->cluster && (g.nt > kMaxClusterTiles || g.X != 0 || h->persistent ||
                      h->smem + 2 * (size_t)g.E * im->value_bytes > (size_t)max_smem)) {
     delete h;
     return SWEPT_EINVAL;
@@ -486,6 +513,10 @@ swept_status swept_init(const swept_config* cfg, swept_handle** out) {
   *out = h;
   return SWEPT_OK;
 }
+
+}  // namespace swept
+
+extern "C" {
 
 swept_status swept_workspace_size(const swept_handle* h, size_t* bytes) {
   if (!h || !bytes) return SWEPT_EINVAL;

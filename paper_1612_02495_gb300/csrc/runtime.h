@@ -46,6 +46,8 @@ struct swept_handle {
 };
 
 namespace swept {
+// swept_init for one of `parts` ranks of a split grid: a default tile leaves each a tile
+swept_status make_plan(const swept_config* cfg, int parts, swept_handle** out);
 // symbolic replay of the swept launch sequence (check.cpp)
 swept_status check_schedule(swept_handle* h, int64_t nsteps, int64_t* computed);
 }  // namespace swept

@@ -46,13 +46,13 @@ swept_status fail(swept_slab* h, swept_status st, const std::string& msg) {
 
 namespace swept {
 
-// The plan of swept_init for cfg, and the slab of `rank`: shared with the
+// The plan for cfg (a default tile leaves each rank one), and the slab of `rank`: shared with the
 // symbolic replay (check.cpp) so both see the same tiling.
 swept_status slab_plan(const swept_config* cfg, int rank, int nranks, Geom* g, Slab* sl, swept_handle** plan_out) {
   if (!cfg || nranks < 1 || rank < 0 || rank >= nranks) return SWEPT_EINVAL;
   if (cfg->persistent != 0 || cfg->cluster != 0) return SWEPT_EUNSUPPORTED;
   swept_handle* h = nullptr;
-  const swept_status st = swept_init(cfg, &h);
+  const swept_status st = make_plan(cfg, nranks, &h);
   if (st != SWEPT_OK) return st;
   if (!h->tiled) {
     swept_free(h);
