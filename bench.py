@@ -73,6 +73,8 @@ WORK = {
            "instr_f64": FP64_INSTR_PER_SUBSTEP, "flops_f64": FP64_FLOPS_PER_SUBSTEP},
     "euler": {"instr": 71, "flops": 82, "smem_acc": 34.5, "instr_f64": 53.5, "flops_f64": 64.5},
     "heat2d": {"instr": 5, "flops": 6, "smem_acc": 6.0},
+    # overlapped tiles: columns in registers, and in FP64 the three sums on the integer pipes
+    "heat2d_tile": {"instr": 5, "flops": 6, "smem_acc": 3.0, "instr_f64": 2, "flops_f64": 3},
 }
 
 
@@ -112,6 +114,8 @@ def dominant_swept_kernel(sol, u, u0, nsteps, solve_ms):
     diamond launches with CUDA events around each (swept_profile_passes)."""
     plan = sol.plan
     units = sol.n * plan["stages"] * nsteps
+    if not sol.cfg.tile_w:
+        return "the library's choice (k_resident on small heat and KS grids)", units, solve_ms, 1.0
     P = plan["tile_w"] // 32 if plan.get("warp_tiles") else 0
     tmpl = "<%s, %s%s>" % ("double" if sol.dtype == 1 else "float",
                           {0: "HeatOp", 1: "KsOp", 2: "EulerOp"}[sol.scheme], ", %d" % P if P else "")
@@ -486,7 +490,7 @@ def measure_sizes(S, autotune, torch, stream, barrier, ws, flush):
         sol.sync_status()
         kname, kunits, kms, share = dominant_swept_kernel(sol, u, d0, nsteps, res["swept"])
         sol.close()
-        rf = alu_roofline(scheme, dt == "f64", kunits, kms, kname, registers=bool(plan.get("warp_tiles")))
+        rf = alu_roofline(scheme, dt == "f64", kunits, kms, kname, registers=bool(plan.get("warp_tiles")) or not plan["tile_w"])
         rf["kernel_share"] = share
         row = {"workload": label, "swept_ms": res["swept"], "classic_ms": res["classic"],
                "speedup_vs_classic": res["classic"] / res["swept"],
@@ -552,9 +556,9 @@ def measure_heat2d(S, autotune, torch, stream, barrier, ws, flush):
         sol.sync_status()
         sol.close()
         pers = plan.get("persistent", 0)
-        kname = ("k_persist2d<%s>" if pers else "k_pyr2d + k_bridge2d + k_octa2d <%s> (the solve's graph)") % (
-            "double" if dt == "f64" else "float")
-        rf = alu_roofline("heat2d", dt == "f64", n * n * nsteps, res["swept"], kname,
+        kname = ("k_persist2d<%s>" if pers else "k_tile2d<%s> (the solve's graph)" if not plan["tile_w"] else
+                 "k_pyr2d + k_bridge2d + k_octa2d <%s> (the solve's graph)") % ("double" if dt == "f64" else "float")
+        rf = alu_roofline("heat2d" if plan["tile_w"] else "heat2d_tile", dt == "f64", n * n * nsteps, res["swept"], kname,
                           note=None if pers else "per-pass plan: the solve's time, launch gaps included")
         out.append({"workload": label, "swept_ms": res["swept"], "classic_ms": res["classic"],
                     "speedup_vs_classic": res["classic"] / res["swept"],

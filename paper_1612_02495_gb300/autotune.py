@@ -9,7 +9,10 @@ and caches the winners in a JSON file keyed by device, scheme, dtype and size.
   tune_single(scheme, dtype, n, ...)  -> {"tile_w", "threads", "warp_tiles", "persistent", "cluster", "ms"}
   tune_batch(problems, dtype, ...)    -> {"tile_w", "threads", "rule", "ms"} for one batch plan
 
-Both only launch the library's kernels through the C ABI.
+Both only launch the library's kernels through the C ABI.  A plan with every
+field 0, the library's choice, is tried too: it may run a kernel that no other
+plan selects.  The number in a cache key goes up with the kernels, so that
+winners among older ones are not kept.
 """
 import json
 import os
@@ -114,11 +117,11 @@ def tune_single(scheme, dtype, n, probe_steps=None, cache=DEFAULT_CACHE, refresh
     `threads`, and (warp_tiles) one warp per tile with the tier rows in
     registers.  Modes: 0 one launch per pass; 1 one persistent kernel; 2 one
     thread-block cluster holding every tile (tried only with at most
-    MAX_CLUSTER_TILES tiles)."""
+    MAX_CLUSTER_TILES tiles).  And the library's choice, a plan with every field 0."""
     import torch
 
     table = _load(cache) if cache else {}
-    key = "single4/%s/%d/%d/%d/%s/%d" % (_device_key(), scheme, dtype, n, probe_steps, int(warp_tiles))
+    key = "single5/%s/%d/%d/%d/%s/%d" % (_device_key(), scheme, dtype, n, probe_steps, int(warp_tiles))
     if not refresh and key in table:
         return table[key]
     u0, args, bc = problem(scheme, dtype, n)
@@ -126,6 +129,22 @@ def tune_single(scheme, dtype, n, probe_steps=None, cache=DEFAULT_CACHE, refresh
     steps = probe_steps or max(64, 4 * h_steps)
     best = None
     d0 = torch.from_numpy(np.ascontiguousarray(u0)).cuda()
+
+    def trial(W, t, mode, wt):
+        nonlocal best
+        try:
+            sol = S.Solver(scheme, dtype, n, *args, bc=bc, tile_w=W, threads=t, persistent=int(mode == 1),
+                           cluster=int(mode == 2), warp_tiles=wt)
+        except S.SweptError:
+            return  # e.g. a cluster window that does not fit in shared memory
+        u = d0.clone()
+        ms = _time(lambda: sol.step(u, steps), reps)
+        sol.close()
+        if best is None or ms < best["ms"]:
+            best = {"tile_w": W, "threads": t, "warp_tiles": wt, "persistent": int(mode == 1),
+                    "cluster": int(mode == 2), "ms": ms, "probe_steps": steps}
+
+    trial(0, 0, 0, 0)
     for W in tile_candidates(scheme, n):
         mappings = [(t, 0) for t in threads if t <= max(32, 2 * W)]
         if warp_tiles and warp_tile_ok(scheme, W, n):
@@ -134,17 +153,7 @@ def tune_single(scheme, dtype, n, probe_steps=None, cache=DEFAULT_CACHE, refresh
             for mode in modes:
                 if mode == 2 and (n // W > MAX_CLUSTER_TILES or n % W):
                     continue
-                try:
-                    sol = S.Solver(scheme, dtype, n, *args, bc=bc, tile_w=W, threads=t, persistent=int(mode == 1),
-                                   cluster=int(mode == 2), warp_tiles=wt)
-                except S.SweptError:
-                    continue  # e.g. a cluster window that does not fit in shared memory
-                u = d0.clone()
-                ms = _time(lambda: sol.step(u, steps), reps)
-                sol.close()
-                if best is None or ms < best["ms"]:
-                    best = {"tile_w": W, "threads": t, "warp_tiles": wt, "persistent": int(mode == 1),
-                            "cluster": int(mode == 2), "ms": ms, "probe_steps": steps}
+                trial(W, t, mode, wt)
     if cache:
         table = _load(cache)
         table[key] = best
@@ -162,30 +171,29 @@ def solver_from_plan(scheme, dtype, n, dx, dt, param0, plan, bc=S.BC_PERIODIC):
 def tune_2d(dtype, nx, ny, probe_steps=200, tiles=(16, 32, 64, 128), threads=(256, 512, 1024), modes=(0, 1),
             cache=DEFAULT_CACHE, refresh=False, reps=2):
     """Best (tile_w, threads, persistent) for swept2d_step_n on an nx x ny 2D heat
-    problem; modes: 0 one launch per pass, 1 the persistent queue kernel."""
+    problem, the library's choice (all 0) among them; modes: 0 one launch per pass, 1 the
+    persistent queue kernel."""
     import torch
 
     table = _load(cache) if cache else {}
-    key = "2d2/%s/%d/%d/%d/%d/%s" % (_device_key(), dtype, nx, ny, probe_steps, "".join(str(m) for m in modes))
+    key = "2d3/%s/%d/%d/%d/%d/%s" % (_device_key(), dtype, nx, ny, probe_steps, "".join(str(m) for m in modes))
     if not refresh and key in table:
         return table[key]
     npd = np.float64 if dtype == S.F64 else np.float32
     p = inputs.heat2d_problem(nx=nx, ny=ny, dtype=npd)
     d0 = torch.from_numpy(p["u0"]).cuda()
     best = None
-    for W in tiles:
-        for t in threads:
-            for m in modes:
-                try:
-                    sol = S.Solver2D(dtype, nx, ny, p["dx"], p["dt"], p["alpha"], tile_w=W, threads=t, persistent=m)
-                except S.SweptError:
-                    continue  # tile not legal for this grid or dtype
-                u = d0.clone()
-                ms = _time(lambda: sol.step(u, probe_steps), reps)
-                sol.sync_status()
-                sol.close()
-                if best is None or ms < best["ms"]:
-                    best = {"tile_w": W, "threads": t, "persistent": m, "ms": ms, "probe_steps": probe_steps}
+    for W, t, m in [(0, 0, 0)] + [(W, t, m) for W in tiles for t in threads for m in modes]:
+        try:
+            sol = S.Solver2D(dtype, nx, ny, p["dx"], p["dt"], p["alpha"], tile_w=W, threads=t, persistent=m)
+        except S.SweptError:
+            continue  # tile not legal for this grid or dtype
+        u = d0.clone()
+        ms = _time(lambda: sol.step(u, probe_steps), reps)
+        sol.sync_status()
+        sol.close()
+        if best is None or ms < best["ms"]:
+            best = {"tile_w": W, "threads": t, "persistent": m, "ms": ms, "probe_steps": probe_steps}
     if cache:
         table = _load(cache)
         table[key] = best
@@ -223,7 +231,7 @@ def tune_batch(problems, dtype, tiles=(128, 256, 512, 1024), threads=(64, 128, 2
 
     sig = (len(problems), int(sum(q["n"] for q in problems)), int(sum(q["nsteps"] for q in problems)))
     table = _load(cache) if cache else {}
-    key = "batch2/%s/%d/%d/%d/%d" % ((_device_key(), dtype) + sig)
+    key = "batch3/%s/%d/%d/%d/%d" % ((_device_key(), dtype) + sig)
     if not refresh and key in table:
         return table[key]
     probe = []
