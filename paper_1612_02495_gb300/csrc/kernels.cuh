@@ -544,25 +544,27 @@ struct FixedTiers {
 // False, with nothing done, when a thread would own more than MAXQ pairs: 4, or
 // 2 out of line (with 4 there, tile 1024 and 128 threads took 1.01 ms where
 // one pair a trip takes 0.96; 8 pairs take 32 registers for the rows alone and
-// lost a third).  ODD: a range may start or end inside a pair (heat; KS with an
+// lost a third).  A single warp of KS: 2, as it walks a narrowing range's pairs one after another here, where
+// the other mapping keeps its lanes together (2^14 points, tile 256, 32 threads, 2,500 steps 2.03 ms with 4, 1.86
+// with 2, 1.82 with none).  ODD: a range may start or end inside a pair (heat; KS with an
 // odd-sized wide tile).
 template <class Op, int MAXQ>
 __device__ __forceinline__ bool fixed_tiers(float* sm, int M, int n, int lo0, int hi0, int d,
                                             const typename Op::K& k) {
   if (!phase_in_window<Op>(M, n, lo0, hi0, d)) return true;
-  const int T = (int)blockDim.x, pairs = (M - 2 * (Op::R & ~1) + 1) / 2, need = (pairs + T - 1) / T;
-  if ((M & 1) || need > MAXQ) return false;
+  const int T = (int)blockDim.x, pairs = (M - 2 * (Op::R & ~1) + 1) / 2;
+  if ((M & 1) || pairs > (Op::R == 2 && T == 32 ? min(MAXQ, 2) : MAXQ) * T) return false;
   if (Op::R == 1 || ((lo0 | hi0) & 1)) {
-    if (need <= 1)
+    if (pairs <= T)
       FixedTiers<Op, 1, true>::run(sm, M, n, lo0, hi0, d, k);
-    else if (need <= 2)
+    else if (pairs <= 2 * T)
       FixedTiers<Op, 2, true>::run(sm, M, n, lo0, hi0, d, k);
     else if constexpr (MAXQ > 2)
       FixedTiers<Op, 4, true>::run(sm, M, n, lo0, hi0, d, k);
   } else if constexpr (Op::R == 2) {
-    if (need <= 1)
+    if (pairs <= T)
       FixedTiers<Op, 1, false>::run(sm, M, n, lo0, hi0, d, k);
-    else if (need <= 2)
+    else if (pairs <= 2 * T)
       FixedTiers<Op, 2, false>::run(sm, M, n, lo0, hi0, d, k);
     else if constexpr (MAXQ > 2)
       FixedTiers<Op, 4, false>::run(sm, M, n, lo0, hi0, d, k);
