@@ -2,6 +2,7 @@
 #pragma once
 #include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "impl.h"
@@ -55,13 +56,24 @@ struct Launch {
     }
     return e;
   }
+  // Threads a KS block in FP64 is launched with: no more than a tier has points.  The integer pipes belong to
+  // a sub-partition each and a block's warps go to them in turn, so with idle warps in every block the working ones
+  // of all blocks meet on the same sub-partitions (2^19 points, 100 steps: tile 32, 64 threads 4.43 ms,
+  // 32 threads 2.39; tile 128, 256 threads 2.26, 128 threads 1.78).  The wide last tile counts, because a
+  // pass that does not fill the GPU lasts as long as its slowest block, unless it doubles the threads of all
+  // tiles on a grid that does.
+  static int used_threads(const Geom& g, int threads) {
+    if (sizeof(T) != 8 || Op::R != 2 || Op::C != 1 || g.P != 0) return threads;
+    const int warps = (g.W + 31) / 32, wide = (g.W + g.X + 31) / 32;
+    return std::min(threads, 32 * (wide >= 2 * warps && g.nt * warps > kKsLoneWarps ? warps : wide));
+  }
   static cudaError_t up(const Geom& g, const void* k, const void* u_in, void* u_out, void* e_out, int hh,
                         int write_top, int threads, size_t smem, cudaStream_t s) {
     return with_p(g.P, [&](auto pc) {
       constexpr int P = decltype(pc)::value;
       return with_maxt<P>(threads, [&](auto mc) {
         constexpr int MAXT = decltype(mc)::value;
-        k_swept_up<T, Op, P, MAXT><<<(unsigned)g.nt, threads, smem, s>>>(g, kc(k), (const T*)u_in, (T*)u_out,
+        k_swept_up<T, Op, P, MAXT><<<(unsigned)g.nt, used_threads(g, threads), smem, s>>>(g, kc(k), (const T*)u_in, (T*)u_out,
                                                                          (T*)e_out, hh, write_top);
         return cudaGetLastError();
       });
@@ -73,7 +85,7 @@ struct Launch {
       constexpr int P = decltype(pc)::value;
       return with_maxt<P>(threads, [&](auto mc) {
         constexpr int MAXT = decltype(mc)::value;
-        k_swept_diamond<T, Op, P, MAXT><<<(unsigned)g.nt, threads, smem, s>>>(g, kc(k), (T*)u_out, (const T*)e_in,
+        k_swept_diamond<T, Op, P, MAXT><<<(unsigned)g.nt, used_threads(g, threads), smem, s>>>(g, kc(k), (T*)u_out, (const T*)e_in,
                                                                               (T*)e_out, odd, mode, hh);
         return cudaGetLastError();
       });
@@ -102,7 +114,7 @@ struct Launch {
         cudaError_t e = raise_smem_limit((const void*)k_swept_persist<T, Op, P, MAXT>, smem);
         if (e != cudaSuccess) return e;
         PersistCtl c{done, queue, error, spin_limit, start_item};
-        k_swept_persist<T, Op, P, MAXT><<<blocks, threads, smem, s>>>(g, kc(k), (T*)u, (T*)e0, (T*)e1, n_sub, c);
+        k_swept_persist<T, Op, P, MAXT><<<blocks, used_threads(g, threads), smem, s>>>(g, kc(k), (T*)u, (T*)e0, (T*)e1, n_sub, c);
         return cudaGetLastError();
       });
     });
@@ -209,7 +221,7 @@ struct Launch {
                              int hh, int write_top, int threads, size_t smem, cudaStream_t s) {
     return with_p(g.P, [&](auto pc) {
       constexpr int P = decltype(pc)::value;
-      k_slab_up<T, Op, P><<<(unsigned)sl.nb, threads, smem, s>>>(g, sl, kc(k), (const T*)u_in, (T*)u_out,
+      k_slab_up<T, Op, P><<<(unsigned)sl.nb, used_threads(g, threads), smem, s>>>(g, sl, kc(k), (const T*)u_in, (T*)u_out,
                                                                   (T*)e_out, hh, write_top);
       return cudaGetLastError();
     });
@@ -218,7 +230,7 @@ struct Launch {
                                   void* e_out, int odd, int mode, int hh, int threads, size_t smem, cudaStream_t s) {
     return with_p(g.P, [&](auto pc) {
       constexpr int P = decltype(pc)::value;
-      k_slab_diamond<T, Op, P><<<(unsigned)sl.nb, threads, smem, s>>>(g, sl, kc(k), (T*)u_out, (const T*)e_in,
+      k_slab_diamond<T, Op, P><<<(unsigned)sl.nb, used_threads(g, threads), smem, s>>>(g, sl, kc(k), (T*)u_out, (const T*)e_in,
                                                                        (T*)e_out, odd, mode, hh);
       return cudaGetLastError();
     });

@@ -355,9 +355,9 @@ struct KsNote {
 };
 constexpr int kKsLoneWarps = 2 * 4 * 152;
 
-// at the start of a pass; FP64 where a thread makes more trips than ks_f64_tier has bits for
-__device__ __forceinline__ void ks_begin(void* row0, const Geom& g) {
-  if (threadIdx.x == 0) *reinterpret_cast<KsNote*>(row0) = KsNote{0, g.W + g.X > 32 * (int)blockDim.x, {}};
+// at the start of a pass; FP64 where a thread makes more trips than ks_f64_tier has bits for, or as the caller says
+__device__ __forceinline__ void ks_begin(void* row0, const Geom& g, bool fp64 = false) {
+  if (threadIdx.x == 0) *reinterpret_cast<KsNote*>(row0) = KsNote{0, fp64 || g.W + g.X > 32 * (int)blockDim.x, {}};
 }
 // one warp's `lost` trips in odd tier s of the pass, on a range of `points`
 __device__ __forceinline__ void ks_note(KsNote* note, unsigned lost, int s, int points, int64_t blocks) {
@@ -876,7 +876,13 @@ struct PDevCtx {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e, edge_slots(g) * g.E, dbg::EDGE)) e_out[e] = row(r, c)[j];
   }
   __device__ __forceinline__ void begin_pass() {
-    if (sizeof(T) == 8) ks_begin(sm, g);
+    // Blocks of one or two warps, with one point a thread or a few blocks in all: the integer chain is the
+    // longer one in this kernel, whose registers are cut to 80 (2^14 points, 1,500 steps: tile 64, 64 threads
+    // 4.44 ms, FP64 4.06; tile 1024 22.2 and 21.3; 2^16, tile 512, 600 steps 5.55 and 6.05)
+    if (sizeof(T) == 8) {
+      const int64_t blocks = min((int64_t)gridDim.x, g.nt);
+      ks_begin(sm, g, blockDim.x <= 64 && blocks * 2 <= (g.W <= (int)blockDim.x ? kKsLoneWarps : kKsLoneWarps / 16));
+    }
   }
   // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
   __device__ __forceinline__ bool phase_tiers(int n, int base, int lo0, int hi0, int d, int64_t , int wall) {
