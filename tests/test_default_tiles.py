@@ -76,3 +76,17 @@ def test_calls_of_before():
     for scheme in (S.HEAT, S.KS):
         for n, dtype in ((1024, S.F32), (512, S.F32), (512, S.F64)):
             S.slab_check(scheme, dtype, n, 0.1, 0.001, 1.0, 8, 7)
+
+
+@pytest.mark.parametrize("scheme,dtype", [(S.HEAT, S.F64), (S.EULER, S.F32), (S.KS, S.F32), (S.KS, S.F64)])
+def test_last_tile(scheme, dtype):
+    """Where no width divides the grid the last tile takes the rest, and every pass waits for it: the widened
+    tile leaves less than a quarter of itself (33,003 points in tiles of 256 left 235)"""
+    for n in (20011, 33003, 48017, 65003):
+        cfg = S.make_config(scheme, dtype, n, 0.1, 0.001, 1.4)
+        h = ctypes.c_void_p()
+        assert S.swept_init(ctypes.byref(cfg), ctypes.byref(h)) == S.SWEPT_OK
+        info = S.swept_plan_info()
+        S.swept_get_plan(h.value, ctypes.byref(info))
+        S.swept_free(h.value)
+        assert 4 * info.last_tile_extra <= info.tile_w, (n, info.tile_w, info.last_tile_extra)
