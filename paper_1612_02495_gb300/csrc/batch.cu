@@ -108,7 +108,7 @@ struct BatchCtx {
       if (phase_in_window<Op>(g.M, n, lo0, hi0, d)) ks_f64_phase(sm, g.M, n, base, lo0, hi0, d, k, gridDim.x, [](int, int, int) {});
       return true;
     } else {
-      return wall == NO_WALL && fixed_tiers<Op, 4>(sm, g.M, n, lo0, hi0, d, k);
+      return wall == NO_WALL && fixed_tiers_call<Op>(g.M, n, lo0, hi0, d, k);
     }
   }
   // the per-problem kernels' tier code (strided, or paired for radius 2)
