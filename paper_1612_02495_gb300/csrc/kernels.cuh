@@ -879,10 +879,12 @@ struct PDevCtx {
   __device__ __forceinline__ void begin_pass() {
     // Blocks of one or two warps, with one point a thread or a few blocks in all: the integer chain is the
     // longer one in this kernel, whose registers are cut to 80 (2^14 points, 1,500 steps: tile 64, 64 threads
-    // 4.44 ms, FP64 4.06; tile 1024 22.2 and 21.3; 2^16, tile 512, 600 steps 5.55 and 6.05)
+    // 4.44 ms, FP64 4.06; tile 1024 22.2 and 21.3; 2^16, tile 512, 600 steps 5.55 and 6.05; 53,248 points,
+    // tile 32, 7.94 and 7.03)
     if (sizeof(T) == 8) {
       const int64_t blocks = min((int64_t)gridDim.x, g.nt);
-      ks_begin(sm, g, blockDim.x <= 64 && blocks * 2 <= (g.W <= (int)blockDim.x ? kKsLoneWarps : kKsLoneWarps / 16));
+      const int64_t most = g.W > (int)blockDim.x ? kKsLoneWarps / 32 : (blockDim.x == 32 ? 3 : 1) * kKsLoneWarps / 2;
+      ks_begin(sm, g, blockDim.x <= 64 && blocks <= most);
     }
   }
   // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
