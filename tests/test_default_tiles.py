@@ -89,4 +89,5 @@ def test_last_tile(scheme, dtype):
         info = S.swept_plan_info()
         S.swept_get_plan(h.value, ctypes.byref(info))
         S.swept_free(h.value)
-        assert 4 * info.last_tile_extra <= info.tile_w, (n, info.tile_w, info.last_tile_extra)
+        if info.tile_w != plain_width(n, 1 if scheme == S.HEAT else 2):
+            assert 4 * info.last_tile_extra <= info.tile_w, (n, info.tile_w, info.last_tile_extra)
