@@ -89,18 +89,20 @@ int choose_tile(int64_t n, int R, int sms) {
   return 0;
 }
 // A width below `narrowest` (at most n / 2, and n / parts where a grid split over ranks needs a
-// tile for each) gives way to the smallest dividing width of up to twice that, or to one of up to
-// a quarter more for which the busiest SM, with a tile in every round and the last one's n mod w points, has
-// the fewest.  With `narrowest` itself and a remainder of 235 points 33,003 points of Euler FP32 took 0.97 ms for
+// tile for each) gives way to a dividing width of up to twice that, else to any of up to
+// a quarter more: the one for which the busiest SM, with a tile in every round and the last one's n mod w points,
+// has the fewest.  With `narrowest` itself and a remainder of 235 points 33,003 points of Euler FP32 took 0.97 ms for
 // 0.86, of heat FP64 0.91 for 0.71.
 int widen_tile(int64_t n, int R, int W, int narrowest, int parts, int sms) {
   const int most = (int)std::min<int64_t>(n / std::max(parts, 2), 1 << 30);
   const int least = std::min(narrowest, most) / (4 * R) * (4 * R);
   if (W == 0 || W >= least) return W;
-  for (int w = least; w <= std::min(2 * least, most); w += 4 * R)
-    if (tile_divides(n, w, R)) return w;
   auto busiest = [&](int w) { return (n / w + sms - 1) / sms * w + n % w; };
-  int best = least;
+  int best = 0;
+  for (int w = least; w <= std::min(2 * least, most); w += 4 * R)
+    if (tile_divides(n, w, R) && (!best || busiest(w) < busiest(best))) best = w;
+  if (best) return best;
+  best = least;
   for (int w = least; w <= std::min(least * 5 / 4, most); w += 4 * R)
     if (busiest(w) < busiest(best)) best = w;
   return best;
