@@ -99,8 +99,8 @@ struct BatchCtx {
   __device__ __forceinline__ void store_edge(int r, int c, int j, int64_t e) {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e, edge_slots(g) * g.E, dbg::EDGE)) e_out[e] = row(r, c)[j];
   }
-  __device__ __forceinline__ void begin_pass() {
-    if (sizeof(T) == 8) ks_begin(sm, g);
+  __device__ __forceinline__ void begin_pass(int w) {
+    if (sizeof(T) == 8) ks_begin(sm, w);
   }
   // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
   __device__ __forceinline__ bool phase_tiers(int n, int base, int lo0, int hi0, int d, int64_t , int wall) {

@@ -335,7 +335,7 @@ __device__ __forceinline__ bool phase_in_window(int M, int n, int lo0, int hi0, 
 //   - A launch that fills the GPU is bound by the FP64 and integer pipes: integers and a second run at some
 //     points cost more than FP64 alone when half of a tier's trips fail.
 //   - With at most two working warps a sub-partition a tier lasts as long as its slowest warp, 970 cycles a
-//     trip or, with a failing point, 2,030, where FP64 alone takes 1,040: one lost trip in eight is too many.
+//     trip or, with a failing point, 2,030, where FP64 alone takes 1,040: one lost trip in four is too many.
 // All of this runs where a point has failed; the others read one word every second tier.  Milliseconds (last:
 // FP64 alone), noisy field and constant one, before and with the count:
 //   2^20, tile 1024, 256 threads, persistent, 400 steps   10.35 / 26.5    10.4 / 18.2    18.3
@@ -356,20 +356,21 @@ struct KsNote {
 constexpr int kKsLoneWarps = 2 * 4 * 152;
 
 // at the start of a pass; FP64 where a thread makes more trips than ks_f64_tier has bits for, or as the caller says
-__device__ __forceinline__ void ks_begin(void* row0, const Geom& g, bool fp64 = false) {
-  if (threadIdx.x == 0) *reinterpret_cast<KsNote*>(row0) = KsNote{0, fp64 || g.W + g.X > 32 * (int)blockDim.x, {}};
+__device__ __forceinline__ void ks_begin(void* row0, int w, bool fp64 = false) {
+  if (threadIdx.x == 0) *reinterpret_cast<KsNote*>(row0) = KsNote{0, fp64 || w > 32 * (int)blockDim.x, {}};
 }
 // one warp's `lost` trips in odd tier s of the pass, on a range of `points`
 __device__ __forceinline__ void ks_note(KsNote* note, unsigned lost, int s, int points, int64_t blocks) {
   const int T = (int)blockDim.x, slot = (s >> 1) & 1;
   note->now[slot ^ 1] = 0;
   const unsigned now = atomicAdd(&note->now[slot], lost) + lost, all = atomicAdd(&note->lost, lost) + lost;
-  const bool lone = (int)min(blocks, (int64_t)kKsLoneWarps + 1) * ((min(T, points) + 31) >> 5) <= kKsLoneWarps;
-  // a single trip may fail on any field, but for the few points of a pass's first tier; a warp makes points / T
-  // trips a tier, at least one, in (s + 1) / 2 odd tiers
-  const unsigned least = s > 1 ? 2 : 1;
-  if (lone ? all >= least && 8 * all * T >= (unsigned)((s + 1) / 2 * max(points, T))
-           : now >= least && 64 * now >= (unsigned)points)
+  const unsigned warps = (unsigned)(min(T, points) + 31) >> 5;
+  const bool lone = (unsigned)min(blocks, (int64_t)kKsLoneWarps + 1) * warps <= (unsigned)kKsLoneWarps;
+  // Few trips may fail on any field, but for those of a pass's first tier, and one block that goes over holds up
+  // a whole pass (2^15 points, tile 256, 610 steps: 1.43 ms, 1.50 with two lost trips, one in eight, enough).  A warp makes
+  // points / T trips a tier, at least one, in (s + 1) / 2 odd tiers.
+  if (lone ? all >= (s > 1 ? 2u + T / 64 : 1u) && 4 * all * T >= (unsigned)((s + 1) / 2 * max(points, T))
+           : now >= (s > 1 ? 4u : 1u) && 64 * now >= (unsigned)points)
     note->fp64 = 1;
 }
 // The points that the integer form did not handle: bit 0 of `failed` is the thread's last trip.  Called by the lanes
@@ -630,8 +631,8 @@ struct DevCtx {
   __device__ __forceinline__ void store_edge(int r, int c, int j, int64_t e) {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e, edge_slots(g) * g.E, dbg::EDGE)) e_out[e] = row(r, c)[j];
   }
-  __device__ __forceinline__ void begin_pass() {
-    if (sizeof(T) == 8) ks_begin(sm, g);
+  __device__ __forceinline__ void begin_pass(int w) {
+    if (sizeof(T) == 8) ks_begin(sm, w);
   }
   // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
   __device__ __forceinline__ bool phase_tiers(int n, int base, int lo0, int hi0, int d, int64_t origin, int wall) {
@@ -876,7 +877,7 @@ struct PDevCtx {
   __device__ __forceinline__ void store_edge(int r, int c, int j, int64_t e) {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e, edge_slots(g) * g.E, dbg::EDGE)) e_out[e] = row(r, c)[j];
   }
-  __device__ __forceinline__ void begin_pass() {
+  __device__ __forceinline__ void begin_pass(int w) {
     // Blocks of one or two warps, with one point a thread or a few blocks in all: the integer chain is the
     // longer one in this kernel, whose registers are cut to 80 (2^14 points, 1,500 steps: tile 64, 64 threads
     // 4.44 ms, FP64 4.06; tile 1024 22.2 and 21.3; 2^16, tile 512, 600 steps 5.55 and 6.05; 53,248 points,
@@ -884,7 +885,7 @@ struct PDevCtx {
     if (sizeof(T) == 8) {
       const int64_t blocks = min((int64_t)gridDim.x, g.nt);
       const int64_t most = g.W > (int)blockDim.x ? kKsLoneWarps / 32 : (blockDim.x == 32 ? 3 : 1) * kKsLoneWarps / 2;
-      ks_begin(sm, g, blockDim.x <= 64 && blocks <= most);
+      ks_begin(sm, w, blockDim.x <= 64 && blocks <= most);
     }
   }
   // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
@@ -1011,8 +1012,8 @@ struct ClusterCtx {
     if (dbg::win(g.M, r, c, kC, j) && dbg::in_range(e - (int64_t)my_rank * g.E, g.E, dbg::EDGE))
       ex_out[e - (int64_t)my_rank * g.E] = row(r, c)[j];
   }
-  __device__ __forceinline__ void begin_pass() {
-    if (sizeof(T) == 8) ks_begin(sm, g);
+  __device__ __forceinline__ void begin_pass(int w) {
+    if (sizeof(T) == 8) ks_begin(sm, w);
   }
   // all tiers of a phase: FP32 with a fixed mapping of points to threads, KS in FP64 (ks_f64_phase)
   __device__ __forceinline__ bool phase_tiers(int n, int base, int lo0, int hi0, int d, int64_t , int wall) {
@@ -1278,7 +1279,7 @@ struct AdjCtx {
     __syncthreads();
   }
   // KS: all tiers of a phase
-  __device__ __forceinline__ void begin_pass() { ks_begin(sm, g); }
+  __device__ __forceinline__ void begin_pass(int w) { ks_begin(sm, w); }
   __device__ __forceinline__ bool phase_tiers(int n, int b, int lo, int hi, int d, int64_t origin, int /*wall*/) {
     if (!phase_in_window<AOp>(g.M, n, lo, hi, d) || !dbg::ok(base + b >= 0 && base + b + n <= top, dbg::TAPE, base + b))
       return true;

@@ -62,7 +62,7 @@ SW_HD void for_tiers(int n, F&& f) {
   if (s <= n) f(s);
 }
 
-// Contexts with kPhaseTiers have begin_pass(), called before the window is filled, and
+// Contexts with kPhaseTiers have begin_pass(w), called before the window of a tile of w points is filled, and
 // phase_tiers(n, base, lo0, hi0, d, origin, wall): all n tiers of a phase at once, or false with nothing done.
 template <class Cx, class = void>
 struct has_phase_tiers : std::false_type {};
@@ -70,8 +70,8 @@ template <class Cx>
 struct has_phase_tiers<Cx, std::enable_if_t<Cx::kPhaseTiers>> : std::true_type {};
 
 template <class Cx>
-SW_HD void begin_pass(Cx& cx) {
-  if constexpr (has_phase_tiers<Cx>::value) cx.begin_pass();
+SW_HD void begin_pass(Cx& cx, int w) {
+  if constexpr (has_phase_tiers<Cx>::value) cx.begin_pass(w);
 }
 
 // all tiers s = 1..n of a phase (sub-timesteps base + s) on [lo0 + d s, hi0 - d s) (d = R
@@ -96,7 +96,7 @@ SW_HD void run_up(Cx& cx, const Geom& g_in, int64_t b, int hh, bool write_top) {
   const int w = tile_width(g, b);
   const int64_t x0 = b * (int64_t)g.W;
   const int64_t origin = x0 - g.R;
-  begin_pass(cx);
+  begin_pass(cx, w);
   cx.for_range(0, w * g.C, [&](int i) {
     const int c = g.C == 1 ? 0 : i / w, k = i - c * w;
     cx.load_u(0, c, g.R + k, x0 + k);
@@ -156,7 +156,7 @@ SW_HD void run_diamond(Cx& cx, const Geom& g_in, int64_t b, int odd, int mode, i
   const int64_t tr = right_tile(g, odd, b);
   const int per_level = g.C * 2 * g.R;
   const int per_side = hh * per_level;
-  begin_pass(cx);
+  begin_pass(cx, w);
   cx.for_range(0, 2 * per_side, [&](int i) {
     const int which = i >= per_side ? 1 : 0;  // 0: right edges of the left tile, 1: left edges of the right tile
     const int rem = i - which * per_side;
