@@ -83,21 +83,10 @@ __device__ __forceinline__ void strided2_level(T* sm, int M, int out_row, int lo
 // point instead of 6.5.  Needs even lo and hi and an even row
 // stride (every KS tier of a tile whose width is a multiple of 8 has even
 // bounds).  Each point is the same Op::point on the same operands.
-template <typename T>
-struct Pair;
-template <>
-struct Pair<float> {
-  using type = float2;
-};
-template <>
-struct Pair<double> {
-  using type = double2;
-};
-
 template <typename T, class Op, int STAGE>
 __device__ __forceinline__ void paired_level(T* sm, int M, int out_row, int lo, int hi, const typename Op::K& k) {
-  static_assert(Op::R == 2, "paired tiers are for radius-2 stencils");
-  using T2 = typename Pair<T>::type;
+  static_assert(Op::R == 2 && sizeof(T) == 4, "paired tiers are for radius-2 stencils in FP32");
+  using T2 = float2;
   const T2* in = reinterpret_cast<const T2*>(sm + (out_row ^ 1) * M);
   T2* out = reinterpret_cast<T2*>(sm + out_row * M);
   for (int jp = (lo >> 1) + (int)threadIdx.x; jp < (hi >> 1); jp += (int)blockDim.x) {
@@ -114,7 +103,8 @@ __device__ __forceinline__ void paired_level(T* sm, int M, int out_row, int lo, 
 template <typename T, class Op, int STAGE>
 __device__ __forceinline__ void scalar_level_any(T* sm, int M, int out_row, int lo, int hi, int wall, int chunk,
                                                  const typename Op::K& k) {
-  if constexpr (Op::R == 2) {
+  // FP32 only: KS tiers in FP64 have their own code (ks_f64_phase)
+  if constexpr (Op::R == 2 && sizeof(T) == 4) {
     if (wall == NO_WALL && chunk <= 1 && ((lo | hi | M) & 1) == 0) {
       paired_level<T, Op, STAGE>(sm, M, out_row, lo, hi, k);
       return;
@@ -160,7 +150,7 @@ __device__ __forceinline__ void euler_face(const T* pr, const T* pu, const T* pp
 // reconstructs p1 + h from cells f-2, f-1, f; side 1 (right) p1 - h from
 // cells f-1, f, f+1, where h = 1/2 minmod(p1 - p0, p2 - p1).  Adding -h is
 // the same IEEE operation as subtracting h, so both sides equal
-// EulerOp::left_side / right_side bit for bit.
+// EulerOp::left_state / right_state (with finish_side) bit for bit.
 template <typename T>
 __device__ __forceinline__ typename EulerOp<T>::Side euler_side(const T* pr, const T* pu, const T* pp, int f,
                                                                 int owner, int wall, int side,

@@ -221,9 +221,13 @@ struct EulerOp {
   // 127 FP64 pipe slots a cell and sub-step took with both sides' speeds, so in
   // FP64 only the faster side's is computed: which it is shows in single
   // precision (from truncated bits, no FP64 instruction) when the estimates differ
-  // by more than 2^-20 of their sum.  An estimate is within 2^-21.3 of its speed:
-  // truncated p, rho and gamma, the product and the quotient give 2^-21.2, halved
-  // by the root; the root, truncated |u| and the sum 2^-23, 2^-23 and 2^-24.
+  // by more than 2^-20 of their sum.  In units of 2^-23: truncated gamma and p make the quotient smaller by 2 and
+  // truncated rho larger by 1, the product's rounding is 1/2 and __fdividef's 2, together 4.5 at most; the root
+  // halves them and adds 1, truncated |u| is within 1 and the sum's rounding 1/2.  So an estimate is within 3.75 units,
+  // 2^-21.1, of its speed, and their difference within 2^-21.1 of the sum of the speeds.  gamma > 1 (swept_init)
+  // keeps the quotient a normal float and makes |u| < 2^-100 nothing beside c.
+  // On smooth flow the sides are closer than that and both speeds are computed, the second out of line
+  // (2^16 cells, one sine wave, 200 steps: 6.81 ms; with both inline and the halvings on the FP64 pipe 7.53).
   // Sides with the same bits have the same speed; everything else computes both.
   __device__ __forceinline__ static T speed_max(const Side& L, const Side& R, const K& k) {
     if constexpr (sizeof(T) == 8) {
