@@ -64,12 +64,13 @@ SMEM_PEAK_GBS = 3.908e13 / 1e9
 # primitives (2 mul, 1 fma, 1 div), a face flux (2 sides x (12 reconstruction ops, 4 for
 # momentum and energy, 1 mul, 1 div, 1 sqrt, 1 add) + 18 for the Rusanov flux), the update of
 # 3 components (avg. 9 ops over the two stages).
-# FP32 heat and KS tiers keep a thread's own pairs in registers: two paired loads and one paired
-# store per pair, 3 values a point.  FP64 (instr_f64, flops_f64): what runs on the FP64 pipe; Euler
+# FP32 tiers that keep a thread's own pairs in registers (fixed_tiers): KS two paired loads and one
+# paired store per pair, 3 values a point; heat two single loads and the paired store, 2.  Tiles with more
+# pairs a thread run KS pairs with three loads (4.5) and strided heat points (4); tier_accesses decides.  FP64 (instr_f64, flops_f64): what runs on the FP64 pipe; Euler
 # without its products with 1/2 (integer) and with one wave speed a face.
 WORK = {
-    "heat": {"instr": 3, "flops": 4, "smem_acc": 4.0, "smem_acc_paired_f32": 3.0},
-    "ks": {"instr": 11, "flops": 18, "smem_acc": 6.5, "smem_acc_paired_f32": 3.0,
+    "heat": {"instr": 3, "flops": 4, "smem_acc": 4.0},
+    "ks": {"instr": 11, "flops": 18, "smem_acc": 6.5,
            "instr_f64": FP64_INSTR_PER_SUBSTEP, "flops_f64": FP64_FLOPS_PER_SUBSTEP},
     "euler": {"instr": 71, "flops": 82, "smem_acc": 34.5, "instr_f64": 53.5, "flops_f64": 64.5},
     "heat2d": {"instr": 5, "flops": 6, "smem_acc": 6.0},
@@ -78,7 +79,28 @@ WORK = {
 }
 
 
-def alu_roofline(scheme, f64, units, ms, kernel, registers=False, note=None):
+def tier_accesses(scheme, f64, tile_w, threads, limit):
+    """Shared-memory values a point and sub-timestep of a tile in shared memory: FP32 heat and KS
+    by whether a thread's pairs fit its registers (at most `limit` of them: 4 per pass, 2 in
+    the persistent, cluster and batch kernels, 2 for KS in a single warp), as the kernels decide."""
+    if f64 or scheme not in ("heat", "ks"):
+        return WORK[scheme]["smem_acc"]
+    R = 1 if scheme == "heat" else 2
+    M = (tile_w + 2 * R + 1) // 2 * 2
+    pairs = (M - 2 * (R & ~1) + 1) // 2
+    if R == 2 and threads == 32:
+        limit = min(limit, 2)
+    fixed = pairs <= limit * threads
+    return (2.0 if fixed else 4.0) if R == 1 else (3.0 if fixed else 4.5)
+
+
+def plan_accesses(sol, scheme):
+    """tier_accesses of a 1D solver's plan"""
+    p = sol.plan
+    return tier_accesses(scheme, sol.dtype == 1, p["tile_w"], p["threads"], 2 if p["persistent"] or p["cluster"] else 4)
+
+
+def alu_roofline(scheme, f64, units, ms, kernel, registers=False, note=None, acc=None):
     """Roofline of a swept kernel that did `units` point-substeps in `ms`: FP pipe
     (flops against the FP64 or FP32 roof) and shared memory (algorithmic accesses
     of the shared-memory tiers against the probed bandwidth; tiers in registers
@@ -90,7 +112,7 @@ def alu_roofline(scheme, f64, units, ms, kernel, registers=False, note=None):
     flops = w.get("flops_f64", w["flops"]) if pipe64 else w["flops"]
     achieved = flops * rate / 1e12
     vb = 8 if f64 else 4
-    acc = w["smem_acc"] if f64 else w.get("smem_acc_paired_f32", w["smem_acc"])
+    acc = w["smem_acc"] if acc is None else acc
     smem_gbs = 0.0 if registers else acc * vb * rate / 1e9
     out = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
            "traffic": None, "kernel": kernel, "kernel_ms": ms, "units": units,
@@ -331,8 +353,9 @@ def measure_fp32(S, inputs, autotune, torch, stream, barrier, ws):
         res[name] = min(ms)
     sol.sync_status()
     kname, kunits, kms, share = dominant_swept_kernel(sol, u, u0, NSTEPS, res["swept"])
+    acc = plan_accesses(sol, "ks")
     sol.close()
-    rf = alu_roofline("ks", False, kunits, kms, kname, registers=bool(t.get("warp_tiles")))
+    rf = alu_roofline("ks", False, kunits, kms, kname, registers=bool(t.get("warp_tiles")), acc=acc)
     rf["kernel_share"] = share
     return {"workload": "KS N=2^20 FP32, 50,000 steps", "tile_w": t["tile_w"], "threads": t["threads"],
             "plan": {k: t.get(k, 0) for k in ("tile_w", "threads", "warp_tiles", "persistent", "cluster")},
@@ -393,7 +416,6 @@ def measure_batch(S, inputs, autotune, torch, stream, barrier, ws, with_f64):
     # point-substeps and flops of the whole batch (heat: 1 sub-step per step, KS: 2)
     heat = spec["kind"] == 0
     units = int((spec["n"] * spec["steps"] * np.where(heat, 1, 2)).sum())
-    smem_ks = {True: WORK["ks"]["smem_acc"], False: WORK["ks"]["smem_acc_paired_f32"]}
     # Runs of more than about 15 s are timed once, their graph capture inside the timed region
     # (a few ms); the FP32 swept batch (about 2 s) gets a warm-up and the best of two.
     # The FP64 tuner probes a narrower candidate set (each FP64 probe takes about 2.4 s).
@@ -428,8 +450,9 @@ def measure_batch(S, inputs, autotune, torch, stream, barrier, ws, with_f64):
         flops = float((spec["n"] * spec["steps"] * np.where(heat, WORK["heat"]["flops"], 2 * ks_flops)).sum())
         rf["achieved"] = flops / (res["swept"] * 1e-3) / 1e12
         rf["frac"] = rf["achieved"] / rf["peak"]
-        smem_acc = float((spec["n"] * spec["steps"] * np.where(heat, WORK["heat"]["smem_acc" if f64 else "smem_acc_paired_f32"],
-                                                                2 * smem_ks[f64])).sum())
+        tile = plan["tile_w"] or (plan.get("rule") or (512, 0))[0]
+        per = {k: tier_accesses(k, f64, tile, plan["threads"], 2) for k in ("heat", "ks")}
+        smem_acc = float((spec["n"] * spec["steps"] * np.where(heat, per["heat"], 2 * per["ks"])).sum())
         sg = smem_acc * (8 if f64 else 4) / (res["swept"] * 1e-3) / 1e9
         rf["smem"].update({"achieved": sg, "frac": sg / SMEM_PEAK_GBS})
         rf["algorithmic_per_unit"] = {"flops": flops / units, "note": "heat and KS point-substeps of the batch"}
@@ -489,8 +512,9 @@ def measure_sizes(S, autotune, torch, stream, barrier, ws, flush):
             res[name] = best
         sol.sync_status()
         kname, kunits, kms, share = dominant_swept_kernel(sol, u, d0, nsteps, res["swept"])
+        acc = plan_accesses(sol, scheme)
         sol.close()
-        rf = alu_roofline(scheme, dt == "f64", kunits, kms, kname, registers=bool(plan.get("warp_tiles")) or not plan["tile_w"])
+        rf = alu_roofline(scheme, dt == "f64", kunits, kms, kname, acc=acc, registers=bool(plan.get("warp_tiles")) or not plan["tile_w"])
         rf["kernel_share"] = share
         row = {"workload": label, "swept_ms": res["swept"], "classic_ms": res["classic"],
                "speedup_vs_classic": res["classic"] / res["swept"],
