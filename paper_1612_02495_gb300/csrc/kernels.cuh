@@ -311,8 +311,8 @@ __device__ __forceinline__ bool phase_in_window(int M, int n, int lo0, int hi0, 
 // that the loop has no branch and a warp's FP64 instructions start before its
 // integer chain has ended: with the branch at each point a lone warp took 1190
 // cycles a point, without 929.
-// Bound: FP64 and integer issue.  2^20 points,
-// tile 1024, 256 threads, persistent, 1,000 steps: 44.6 -> 26.0 ms.  Two points
+// Bound: FP64 and integer issue (68 % and 74 % of their pipes).  2^20 points,
+// tile 1024, 256 threads, persistent, 1,000 steps: 44.6 -> 25.8 ms.  Two points
 // a thread, sharing their operands' conversions, gave 25.3 ms there but took
 // 2^14 points (tile 128) from 3.85 to 4.22 ms (start: 4.06 ms); four spilled (36.6 ms); four or
 // five blocks a SM instead of three 27.2 and 28.3 ms.
