@@ -50,7 +50,7 @@ DIAMOND_TRAFFIC_BYTES = None
 # the same for one k_swept_persist<double, KsOp> launch (a whole 50,000-step solve), per plan
 # (tile, threads): dram__bytes_read.sum + dram__bytes_write.sum from an ncu capture of just those
 # two counters and the duration, on the current kernel; a plan without a capture reports None
-PERSIST_TRAFFIC = {(1024, 256): 9350400 + 11572224}
+PERSIST_TRAFFIC = {(1024, 256): 9438720 + 13622016}
 
 
 # Measured unit ceilings of GB300 (python -m paper_1612_02495_gb300.peaks, register-only probe loops):
